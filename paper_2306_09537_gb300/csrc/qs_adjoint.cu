@@ -30,6 +30,12 @@ namespace qsk {
 
 constexpr int ADJ_BLOCK_MAX = 256;
 constexpr int NSUB = 29;
+// floats per drone of the backward kernels' shared memory: staged positions
+// (4 each) of both groups, then smooth: lambda of the acceleration (3) and two
+// segments' final position and motor noise (14); discrete: velocities of both
+// groups (6), lambda of the post-collision velocity (3) and, event time,
+// position (3), lambda x' . D and earliest partner
+constexpr int BWD_PLANES = 25;
 // steps of a checkpoint segment whose collision responses the backward records
 constexpr int RFLAG_WORDS = 32, RFLAG_BITS = 32 * RFLAG_WORDS;  // floats of a saved substep input: x v R w wlo uf eps
 
@@ -52,13 +58,14 @@ __device__ __forceinline__ void wall_dacc(const Consts& c, const float x[3], flo
 }
 
 // lambda_x += sum_j J_ij (lam_a_i - lam_a_j)
-__device__ __forceinline__ void pair_vjp(const Consts& c, const float x[3], const float la[3], const float* sx,
+__device__ __forceinline__ void pair_vjp(const Consts& c, const float x[3], const float la[3], const float4* sp,
                                          const float* sla, int nt, int sbase, int lane, int N, float arm, float lx[3]) {
     const float kcg = c.kc * c.g, b = c.beta, far2 = pair_far_d2(arm, c.inv_beta);
     for (int j = 0; j < N; ++j) {
         if (j == lane) continue;
         const int tj = sbase + j;
-        const float r0 = x[0] - sx[tj], r1 = x[1] - sx[nt + tj], r2 = x[2] - sx[2 * nt + tj];
+        const float4 xj = sp[tj];
+        const float r0 = x[0] - xj.x, r1 = x[1] - xj.y, r2 = x[2] - xj.z;
         const float d2 = r0 * r0 + r1 * r1 + r2 * r2;
         if (d2 == 0.f || d2 > far2) continue;
         const float d = sqrtf(d2), id = rcp_approx(d);
@@ -339,16 +346,12 @@ __device__ __forceinline__ bool group_sync_or(int id, int n, bool v) {
 // the substep start, staged in shared memory at the thread's group-local
 // index lt; bid, bn: the barrier of the threads sharing them).
 __device__ __forceinline__ void smooth_substep(const Consts& c, Drone& s, const Prm& p, const float u[4], uint32_t tick,
-                                               int d, int sub, bool act, float* sx, int nt, int sbase, int lane, int N,
+                                               int d, int sub, bool act, float4* sp, int sbase, int lane, int N,
                                                int lt, int bid, int bn, const float* nrm = nullptr) {
-    if (act) {
-        sx[lt] = s.x[0];
-        sx[nt + lt] = s.x[1];
-        sx[2 * nt + lt] = s.x[2];
-    }
+    if (act) sp[lt] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
     group_sync(bid, bn);
     float pa[3] = {0.f, 0.f, 0.f};
-    if (act) pair_acc(c, s.x, sx, nt, sbase, lane, N, p.arm, pa);
+    if (act) pair_acc(c, s.x, sp, sbase, lane, N, p.arm, pa);
     group_sync(bid, bn);
     if (act) substep<false, 1>(s, p, c, u, tick, d, sub, pa, nrm);
 }
@@ -409,7 +412,8 @@ __device__ __forceinline__ void command4(const Consts& c, const float* act, size
 
 __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                             const int* __restrict__ perm, const DiffArgs a) {
-    extern __shared__ float sm[];
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
     const int nb = blockDim.x >> 1, grp = threadIdx.x >= nb ? 1 : 0, lt = threadIdx.x - grp * nb;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, nb);
     const int W = tile.W, nt = nb;
@@ -420,7 +424,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
     const bool ahead = (c.flags & QS_F_MOTOR_NOISE) && c.substeps <= FWD_SUB;
-    float* nbase = sm + 9 * nb;  // [2][FWD_SUB][4][nb] motor normals
+    float4* sp = sm4;            // [nb] positions; then [3][nb] velocities of the collision pass
+    float* nbase = sm + 7 * nb;  // [2][FWD_SUB][4][nb] motor normals
     const uint32_t tick0 = act ? dv.tick[e] : 0u;
     if (grp == 1) {
         fwd_noise_group(c, nbase, nb, lt, act, ahead, tick0, d, a.T);
@@ -451,7 +456,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
             float n[4];
             if (ahead)
                 for (int r = 0; r < 4; ++r) n[r] = *fwd_normals(nbase, nb, t & 1, sub, r, lt);
-            smooth_substep(c, s, p, u, tick0 + t, d, sub, act, sm, nt, sbase, lane, N, lt, 1, nb, ahead ? n : nullptr);
+            smooth_substep(c, s, p, u, tick0 + t, d, sub, act, sp, sbase, lane, N, lt, 1, nb, ahead ? n : nullptr);
         }
         if (act) {
             const float dx = s.x[0] - g[0], dy = s.x[1] - g[1], dz = s.x[2] - g[2];
@@ -475,7 +480,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
 // next saved input instead of drawing it again.
 __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                             const int* __restrict__ perm, const DiffArgs a) {
-    extern __shared__ float sm[];
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
     const int nb = blockDim.x >> 1, grp = threadIdx.x >= nb ? 1 : 0, lt = threadIdx.x - grp * nb, bid = 1 + grp;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, nb);
     const int W = tile.W, nt = nb;
@@ -485,9 +491,9 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, cons
     const bool act = lane < N;
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
-    float* sx = sm + grp * 3 * nb;  // [3][nb] positions of the group
-    float* sla = sm + 6 * nb;       // [3][nb] lambda of the acceleration (group 1)
-    float* fin = sm + 9 * nb;       // [2][7][nb] position and motor noise at the end of a recomputed segment
+    float4* sp = sm4 + grp * nb;  // [nb] positions of the group
+    float* sla = sm + 8 * nb;       // [3][nb] lambda of the acceleration (group 1)
+    float* fin = sm + 11 * nb;      // [2][7][nb] position and motor noise at the end of a recomputed segment
     const int S = c.substeps;
     const size_t sbuf = (size_t)a.C * (S + 1) * NSUB * D;  // floats of one scratch buffer (each substep's input)
     Prm p;
@@ -522,7 +528,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, cons
                 if (act) command4(c, a.act, D, t, d, fh, u, msk);
                 for (int sub = 0; sub < S; ++sub) {
                     if (act) save_sub(scr, D, (t - tb) * S + sub, d, s);
-                    smooth_substep(c, s, p, u, tick0 + t, d, sub, act, sx, nt, sbase, lane, N, lt, bid, nb);
+                    smooth_substep(c, s, p, u, tick0 + t, d, sub, act, sp, sbase, lane, N, lt, bid, nb);
                 }
             }
             if (act) {
@@ -562,11 +568,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, cons
                         else
                             for (int r = 0; r < 4; ++r) eps1[r] = eps_end[r];
                     }
-                    if (act) {
-                        sx[lt] = si.x[0];
-                        sx[nt + lt] = si.x[1];
-                        sx[2 * nt + lt] = si.x[2];
-                    }
+                    if (act) sp[lt] = make_float4(si.x[0], si.x[1], si.x[2], 0.f);
                     group_sync(bid, nb);
                     float la[3] = {0.f, 0.f, 0.f};
                     if (act) {
@@ -576,7 +578,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, cons
                         sla[2 * nt + lt] = la[2];
                     }
                     group_sync(bid, nb);
-                    if (act) pair_vjp(c, si.x, la, sx, sla, nt, sbase, lane, N, p.arm, lx);
+                    if (act) pair_vjp(c, si.x, la, sp, sla, nt, sbase, lane, N, p.arm, lx);
                     group_sync(bid, nb);
                 }
                 if (act) {
@@ -851,17 +853,15 @@ __device__ __forceinline__ void discrete_substep_vjp(const Drone& s, const Prm& 
 }
 
 // The collision pass of a control step (S9, S10) as the step kernels run it:
-// positions and pre-collision velocities staged in shared memory (sx, sv:
-// [3][nt]). Every thread of the CTA calls it.
+// positions and pre-collision velocities staged in shared memory (sp: [nt]
+// float4, sv: [3][nt]). Every thread of the CTA calls it.
 // Returns whether any drone of the group responded (the same value in every
 // thread of the group).
 __device__ __forceinline__ bool discrete_collisions(const Consts& c, Drone& s, const Prm& p, uint32_t tick, int d,
-                                                    bool act, float* sx, float* sv, int nt, int sbase, int lane, int N,
+                                                    bool act, float4* sp, float* sv, int nt, int sbase, int lane, int N,
                                                     int lt, int bid, int bn) {
     if (act) {
-        sx[lt] = s.x[0];
-        sx[nt + lt] = s.x[1];
-        sx[2 * nt + lt] = s.x[2];
+        sp[lt] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
         sv[lt] = s.v[0];
         sv[nt + lt] = s.v[1];
         sv[2 * nt + lt] = s.v[2];
@@ -871,10 +871,10 @@ __device__ __forceinline__ bool discrete_collisions(const Consts& c, Drone& s, c
     bool responded = false;
     if (act && N > 1) {
         uint32_t ev = 0;
-        uint64_t best[QS_MAX_K];
+        NbrList nbrs;
         float az = 0.f;
         bool dwh = false;
-        responded = pair_scan(c, s, p.thr, lane, N, sbase, sx, sv, nt, 0, true, true, ev, best, dvs, false, az, dwh);
+        responded = pair_scan<false>(c, s, p.thr, lane, N, sbase, sp, sv, nt, 0, true, true, ev, nbrs, dvs, false, az, dwh);
     }
     const bool any = group_sync_or(bid, bn, responded);
     if (responded) apply_response(c, s, tick, d, dvs);
@@ -920,12 +920,10 @@ __device__ __forceinline__ PairEt pair_et(const float dx[3], float key, float th
 // The event-time collision pass of a control step (forward); returns whether
 // any drone of the group responded (the same value in every thread of it).
 __device__ __forceinline__ bool discrete_collisions_et(const Consts& c, Drone& s, const Prm& p, uint32_t tick, int d,
-                                                       bool act, float* sx, float* sv, int nt, int sbase, int lane,
+                                                       bool act, float4* sp, float* sv, int nt, int sbase, int lane,
                                                        int N, int lt, int bid, int bn) {
     if (act) {
-        sx[lt] = s.x[0];
-        sx[nt + lt] = s.x[1];
-        sx[2 * nt + lt] = s.x[2];
+        sp[lt] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
         sv[lt] = s.v[0];
         sv[nt + lt] = s.v[1];
         sv[2 * nt + lt] = s.v[2];
@@ -939,7 +937,8 @@ __device__ __forceinline__ bool discrete_collisions_et(const Consts& c, Drone& s
             if (j == lane) continue;
             const int tj = sbase + j;
             float dx[3];
-            const float key = pair_key(s.x[0], s.x[1], s.x[2], sx[tj], sx[nt + tj], sx[2 * nt + tj], dx[0], dx[1], dx[2]);
+            const float4 xj = sp[tj];
+            const float key = pair_key(s.x[0], s.x[1], s.x[2], xj.x, xj.y, xj.z, dx[0], dx[1], dx[2]);
             if (!(key < p.thr)) continue;
             const float rv[3] = {s.v[0] - sv[tj], s.v[1] - sv[nt + tj], s.v[2] - sv[2 * nt + tj]};
             const float app = -dot3(rv[0], rv[1], rv[2], dx[0], dx[1], dx[2]);
@@ -969,7 +968,7 @@ __device__ __forceinline__ bool discrete_collisions_et(const Consts& c, Drone& s
 }
 
 // Adjoint of the collision pass: xs, vs the pre-collision position and
-// velocity of the thread's drone (as staged: sx, sv), sl the lambda of every
+// velocity of the thread's drone (as staged: sp, sv), sl the lambda of every
 // drone's post-collision velocity. For a responding drone i,
 //   v_i' = alpha_c (v_i + sum_j ((v_j - v_i) . n_ij) n_ij + eps),
 //   n_ij = (x_i - x_j) / d_ij,
@@ -978,7 +977,7 @@ __device__ __forceinline__ bool discrete_collisions_et(const Consts& c, Drone& s
 // q = lambda_v_i' - lambda_v_j', P = I - n n^T, vn = (v_j - v_i) . n
 // (the partner relation is symmetric, so every partner also responded).
 __device__ __forceinline__ void collision_vjp(const Consts& c, const float xs[3], const float vs[3], float thr,
-                                              const float* sx, const float* sv, const float* sl, int nt, int sbase,
+                                              const float4* sp, const float* sv, const float* sl, int nt, int sbase,
                                               int lane, int N, float lx[3], float lv[3]) {
     const float l0[3] = {lv[0], lv[1], lv[2]};
     float acc_v[3] = {0.f, 0.f, 0.f}, acc_x[3] = {0.f, 0.f, 0.f};
@@ -987,7 +986,8 @@ __device__ __forceinline__ void collision_vjp(const Consts& c, const float xs[3]
         if (j == lane) continue;
         const int tj = sbase + j;
         float dx, dy, dz;
-        const float key = pair_key(xs[0], xs[1], xs[2], sx[tj], sx[nt + tj], sx[2 * nt + tj], dx, dy, dz);
+        const float4 xj = sp[tj];
+        const float key = pair_key(xs[0], xs[1], xs[2], xj.x, xj.y, xj.z, dx, dy, dz);
         if (!(key < thr)) continue;
         const float rv0 = vs[0] - sv[tj], rv1 = vs[1] - sv[nt + tj], rv2 = vs[2] - sv[2 * nt + tj];
         if (!(-dot3(rv0, rv1, rv2, dx, dy, dz) < 0.0f)) continue;  // approaching
@@ -1040,14 +1040,12 @@ __device__ __forceinline__ void loss_term(float dl, const float x[3], const floa
 // The partners' lambdas, lambda x' . D and earliest partners are exchanged
 // through shared memory (sl, slx, sq, sarg: [3][nt], [3][nt], [nt], [nt]).
 __device__ __forceinline__ void collision_vjp_et(const Consts& c, const Drone& sc, const Prm& p, uint32_t tick, int d,
-                                                 bool act, float* sx, float* sv, float* sl, float* slx, float* sq,
+                                                 bool act, float4* sp, float* sv, float* sl, float* slx, float* sq,
                                                  int* sarg, int nt, int sbase, int lane, int N, int lt, int bid, int bn,
                                                  float dl, const float g[3], float lx[3], float lv[3]) {
     const float Tc = c.substeps * c.dt, ac = c.alpha_c;
     if (act) {
-        sx[lt] = sc.x[0];
-        sx[nt + lt] = sc.x[1];
-        sx[2 * nt + lt] = sc.x[2];
+        sp[lt] = make_float4(sc.x[0], sc.x[1], sc.x[2], 0.f);
         sv[lt] = sc.v[0];
         sv[nt + lt] = sc.v[1];
         sv[2 * nt + lt] = sc.v[2];
@@ -1061,8 +1059,8 @@ __device__ __forceinline__ void collision_vjp_et(const Consts& c, const Drone& s
             if (j == lane) continue;
             const int tj = sbase + j;
             float dx[3];
-            const float key = pair_key(sc.x[0], sc.x[1], sc.x[2], sx[tj], sx[nt + tj], sx[2 * nt + tj], dx[0], dx[1],
-                                       dx[2]);
+            const float4 xj = sp[tj];
+            const float key = pair_key(sc.x[0], sc.x[1], sc.x[2], xj.x, xj.y, xj.z, dx[0], dx[1], dx[2]);
             if (!(key < p.thr)) continue;
             const float rv[3] = {sc.v[0] - sv[tj], sc.v[1] - sv[nt + tj], sc.v[2] - sv[2 * nt + tj]};
             const float app = -dot3(rv[0], rv[1], rv[2], dx[0], dx[1], dx[2]);
@@ -1109,8 +1107,8 @@ __device__ __forceinline__ void collision_vjp_et(const Consts& c, const Drone& s
             if (j == lane) continue;
             const int tj = sbase + j;
             float dx[3];
-            const float key = pair_key(sc.x[0], sc.x[1], sc.x[2], sx[tj], sx[nt + tj], sx[2 * nt + tj], dx[0], dx[1],
-                                       dx[2]);
+            const float4 xj = sp[tj];
+            const float key = pair_key(sc.x[0], sc.x[1], sc.x[2], xj.x, xj.y, xj.z, dx[0], dx[1], dx[2]);
             if (!(key < p.thr)) continue;
             const float rv[3] = {sc.v[0] - sv[tj], sc.v[1] - sv[nt + tj], sc.v[2] - sv[2 * nt + tj]};
             const float app = -dot3(rv[0], rv[1], rv[2], dx[0], dx[1], dx[2]);
@@ -1149,7 +1147,8 @@ __device__ __forceinline__ void collision_vjp_et(const Consts& c, const Drone& s
 template <bool ET>
 __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                              const int* __restrict__ perm, const DiffArgs a) {
-    extern __shared__ float sm[];
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
     const int nb = blockDim.x >> 1, grp = threadIdx.x >= nb ? 1 : 0, lt = threadIdx.x - grp * nb;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, nb);
     const int W = tile.W, nt = nb;
@@ -1161,7 +1160,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
     const size_t D = dv.D;
     const bool coll = (c.flags & QS_F_COLLISIONS) != 0;
     const bool ahead = (c.flags & QS_F_MOTOR_NOISE) && c.substeps <= FWD_SUB;
-    float* nbase = sm + 9 * nb;  // [2][FWD_SUB][4][nb] motor normals
+    float4* sp = sm4;            // [nb] positions; then [3][nb] velocities of the collision pass
+    float* nbase = sm + 7 * nb;  // [2][FWD_SUB][4][nb] motor normals
     const uint32_t tick0 = act ? dv.tick[e] : 0u;
     if (grp == 1) {
         fwd_noise_group(c, nbase, nb, lt, act, ahead, tick0, d, a.T);
@@ -1197,8 +1197,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
                 substep<ET, 0>(s, p, c, u, tick0 + t, d, sub, zero3, ahead ? n : nullptr);
             }
         }
-        if (coll && ET) discrete_collisions_et(c, s, p, tick0 + t, d, act, sm, sm + 3 * nt, nt, sbase, lane, N, lt, 1, nb);
-        else if (coll) discrete_collisions(c, s, p, tick0 + t, d, act, sm, sm + 3 * nt, nt, sbase, lane, N, lt, 1, nb);
+        if (coll && ET) discrete_collisions_et(c, s, p, tick0 + t, d, act, sp, sm + 4 * nt, nt, sbase, lane, N, lt, 1, nb);
+        else if (coll) discrete_collisions(c, s, p, tick0 + t, d, act, sp, sm + 4 * nt, nt, sbase, lane, N, lt, 1, nb);
         if (act) {
             const float dx = s.x[0] - g[0], dy = s.x[1] - g[1], dz = s.x[2] - g[2];
             L += dx * dx + dy * dy + dz * dz + 1e-3f * (fh[0] * fh[0] + fh[1] * fh[1] + fh[2] * fh[2] + fh[3] * fh[3]);
@@ -1217,7 +1217,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
 template <bool ET>
 __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                              const int* __restrict__ perm, const DiffArgs a) {
-    extern __shared__ float sm[];
+    extern __shared__ float4 sm4[];
+    float* sm = reinterpret_cast<float*>(sm4);
     const int nb = blockDim.x >> 1, grp = threadIdx.x >= nb ? 1 : 0, lt = threadIdx.x - grp * nb, bid = 1 + grp;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, nb);
     const int W = tile.W, nt = nb;
@@ -1228,17 +1229,17 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
     const bool coll = (c.flags & QS_F_COLLISIONS) != 0;
-    float* sx = sm + grp * 6 * nb;       // [3][nb] positions of the group
-    float* sv = sx + 3 * nb;             // [3][nb] velocities of the group
-    float* sl = sm + 12 * nb;            // [3][nb] lambda of the post-collision velocity (group 1)
-    float* slx = sm + 15 * nb;           // event time: [3][nb] lambda of the post-collision position,
-    float* sq = sm + 18 * nb;            //   [nb] lambda x' . D, [nb] earliest partner (group 1)
-    int* sarg = reinterpret_cast<int*>(sm + 19 * nb);
+    float4* sp = sm4 + grp * nb;         // [nb] positions of the group
+    float* sv = sm + (8 + grp * 3) * nb; // [3][nb] velocities of the group
+    float* sl = sm + 14 * nb;            // [3][nb] lambda of the post-collision velocity (group 1)
+    float* slx = sm + 17 * nb;           // event time: [3][nb] lambda of the post-collision position,
+    float* sq = sm + 20 * nb;            //   [nb] lambda x' . D, [nb] earliest partner (group 1)
+    int* sarg = reinterpret_cast<int*>(sm + 21 * nb);
     // [2][RFLAG_WORDS] bit q: some drone of the group responded to a collision
     // in step tb + q of the segment recomputed into that buffer (steps beyond
     // RFLAG_BITS are taken as responding); the reverse skips the collision
     // adjoint of a step without responses, which is then the identity
-    uint32_t* rflag = reinterpret_cast<uint32_t*>(sm + 23 * nb);
+    uint32_t* rflag = reinterpret_cast<uint32_t*>(sm + BWD_PLANES * nb);
     const int S = c.substeps, S1 = c.substeps + 1;  // saved states per step: each substep's input, then the pre-collision state
     const size_t sbuf = (size_t)a.C * S1 * NSUB * D;  // floats of one scratch buffer
     Prm p;
@@ -1284,9 +1285,9 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
                 }
                 bool any = false;
                 if (coll && ET)
-                    any = discrete_collisions_et(c, s, p, tick0 + t, d, act, sx, sv, nt, sbase, lane, N, lt, bid, nb);
+                    any = discrete_collisions_et(c, s, p, tick0 + t, d, act, sp, sv, nt, sbase, lane, N, lt, bid, nb);
                 else if (coll)
-                    any = discrete_collisions(c, s, p, tick0 + t, d, act, sx, sv, nt, sbase, lane, N, lt, bid, nb);
+                    any = discrete_collisions(c, s, p, tick0 + t, d, act, sp, sv, nt, sbase, lane, N, lt, bid, nb);
                 if (lt == 0 && any && t - tb < RFLAG_BITS) fl[(t - tb) >> 5] |= 1u << ((t - tb) & 31);
             }
         } else if (grp == 1 && it >= 1) {
@@ -1307,13 +1308,11 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
                     if (!(ET && coll && any)) loss_term(dl, sc.x, g, lx);
                 }
                 if (coll && ET && any) {
-                    collision_vjp_et(c, sc, p, tick0 + t, d, act, sx, sv, sl, slx, sq, sarg, nt, sbase, lane, N, lt, bid,
+                    collision_vjp_et(c, sc, p, tick0 + t, d, act, sp, sv, sl, slx, sq, sarg, nt, sbase, lane, N, lt, bid,
                                      nb, dl, g, lx, lv);
                 } else if (coll && any) {
                     if (act) {
-                        sx[lt] = sc.x[0];
-                        sx[nt + lt] = sc.x[1];
-                        sx[2 * nt + lt] = sc.x[2];
+                        sp[lt] = make_float4(sc.x[0], sc.x[1], sc.x[2], 0.f);
                         sv[lt] = sc.v[0];
                         sv[nt + lt] = sc.v[1];
                         sv[2 * nt + lt] = sc.v[2];
@@ -1322,7 +1321,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
                         sl[2 * nt + lt] = lv[2];
                     }
                     group_sync(bid, nb);
-                    if (act && N > 1) collision_vjp(c, sc.x, sc.v, p.thr, sx, sv, sl, nt, sbase, lane, N, lx, lv);
+                    if (act && N > 1) collision_vjp(c, sc.x, sc.v, p.thr, sp, sv, sl, nt, sbase, lane, N, lx, lv);
                     group_sync(bid, nb);
                 }
                 float lu[4] = {0.f, 0.f, 0.f, 0.f};
@@ -1374,12 +1373,9 @@ cudaError_t launch_diff(int backward, const Consts& c, const Dev& dv, const Tile
     a.ckpt = reinterpret_cast<float4*>(workspace);
     a.scratch = reinterpret_cast<float*>(reinterpret_cast<char*>(workspace) + (size_t)nck * NPLANE * dv.D * sizeof(float4));
     // forward: two groups of `block` threads (integration, motor normals ahead);
-    // backward: two (recompute, reverse) with up to 23 planes of `block` floats
-    // (positions and velocities of both groups, the reverse's lambdas of the
-    // post-collision velocity and, with event-time contacts, position, its
-    // lambda x' . D and earliest partner: 20 planes)
-    const size_t smem = sizeof(float) * (9 + 2 * FWD_SUB * 4) * block,
-                 smem2 = sizeof(float) * 23 * block + sizeof(uint32_t) * 2 * RFLAG_WORDS;
+    // backward: two (recompute, reverse) with BWD_PLANES planes of `block` floats
+    const size_t smem = sizeof(float) * (7 + 2 * FWD_SUB * 4) * block,
+                 smem2 = sizeof(float) * BWD_PLANES * block + sizeof(uint32_t) * 2 * RFLAG_WORDS;
     if (2 * block > ADJ_BLOCK_MAX) return cudaErrorInvalidValue;
     if (c.flags & QS_F_SMOOTH) {
         if (backward) k_diff_bwd<<<n_tiles, 2 * block, smem2, st>>>(c, dv, tiles, perm, a);

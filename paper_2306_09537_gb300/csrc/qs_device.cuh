@@ -458,15 +458,16 @@ __device__ __forceinline__ float pair_far_d2(float arm, float inv_beta) {
 }
 
 // Smooth pair acceleration of the thread's drone from the slot's positions in
-// shared memory (sx[3][nt]); j == lane and coincident drones contribute 0.
-__device__ __forceinline__ void pair_acc(const Consts& c, const float x[3], const float* sx, int nt, int sbase, int lane,
-                                         int N, float arm, float out[3]) {
+// shared memory (sp: one float4 a drone); j == lane and coincident drones
+// contribute 0.
+__device__ __forceinline__ void pair_acc(const Consts& c, const float x[3], const float4* sp, int sbase, int lane, int N,
+                                         float arm, float out[3]) {
     out[0] = out[1] = out[2] = 0.f;
     const float kcg = __fmul_rn(c.kc, c.g), far2 = pair_far_d2(arm, c.inv_beta);
     for (int j = 0; j < N; ++j) {
         if (j == lane) continue;
-        const int tj = sbase + j;
-        const float r0 = x[0] - sx[tj], r1 = x[1] - sx[nt + tj], r2 = x[2] - sx[2 * nt + tj];
+        const float4 q = sp[sbase + j];
+        const float r0 = x[0] - q.x, r1 = x[1] - q.y, r2 = x[2] - q.z;
         const float d2 = __fmaf_rn(r2, r2, __fmaf_rn(r1, r1, __fmul_rn(r0, r0)));
         if (d2 == 0.f || d2 > far2) continue;
         const float d = sqrtf(d2);
@@ -738,41 +739,17 @@ __device__ __forceinline__ float pair_key(float xi0, float xi1, float xi2, float
     return __fadd_rn(__fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)), __fmul_rn(dz, dz));
 }
 
-// Inserts cand into the ascending list best[0..K).
-__device__ __forceinline__ void topk_insert(uint64_t best[QS_MAX_K], int K, uint64_t cand) {
-#pragma unroll
-    for (int k = 0; k < QS_MAX_K; ++k) {
-        if (k < K && cand < best[k]) {
-            const uint64_t t = best[k];
-            best[k] = cand;
-            cand = t;
-        }
-    }
-}
-
-// The same with the list length KN fixed at compile time (no test of k < K).
-template <int KN>
-__device__ __forceinline__ void topk_insert_n(uint64_t best[QS_MAX_K], uint64_t cand) {
-#pragma unroll
-    for (int k = 0; k < KN; ++k) {
-        if (cand < best[k]) {
-            const uint64_t t = best[k];
-            best[k] = cand;
-            cand = t;
-        }
-    }
-}
-
-// Compare-exchange of two (key, index) words: a <- min, b <- max.
-__device__ __forceinline__ void cmp_swap(uint64_t& a, uint64_t& b) {
-    const uint64_t lo = a < b ? a : b, hi = a < b ? b : a;
+// Compare-exchange of two words: a <- min, b <- max.
+template <class T>
+__device__ __forceinline__ void cmp_swap(T& a, T& b) {
+    const T lo = a < b ? a : b, hi = a < b ? b : a;
     a = lo;
     b = hi;
 }
 
 // Sorts k[0..8) ascending with Floyd's 19-comparator network for 8 inputs
 // (Knuth, The Art of Computer Programming vol. 3, Sec. 5.3.4), depth 6:
-// the words are distinct (the low half is the partner index), so the result
+// the words are distinct (the low bits are the partner index), so the result
 // is the same order an insertion sort gives.
 static_assert(QS_MAX_K == 8, "the sorting network holds QS_MAX_K words");
 __device__ __forceinline__ void sort8(uint64_t k[8]) {
@@ -783,15 +760,52 @@ __device__ __forceinline__ void sort8(uint64_t k[8]) {
     cmp_swap(k[1], k[4]); cmp_swap(k[3], k[6]);
     cmp_swap(k[1], k[2]); cmp_swap(k[3], k[4]); cmp_swap(k[5], k[6]);
 }
+__device__ __forceinline__ void sort8(uint32_t k[8]) {
+    cmp_swap(k[0], k[2]); cmp_swap(k[1], k[3]); cmp_swap(k[4], k[6]); cmp_swap(k[5], k[7]);
+    cmp_swap(k[0], k[4]); cmp_swap(k[1], k[5]); cmp_swap(k[2], k[6]); cmp_swap(k[3], k[7]);
+    cmp_swap(k[0], k[1]); cmp_swap(k[2], k[3]); cmp_swap(k[4], k[5]); cmp_swap(k[6], k[7]);
+    cmp_swap(k[2], k[4]); cmp_swap(k[3], k[5]);
+    cmp_swap(k[1], k[4]); cmp_swap(k[3], k[6]);
+    cmp_swap(k[1], k[2]); cmp_swap(k[3], k[4]); cmp_swap(k[5], k[6]);
+}
+// Sorts k[0..4): 5 comparators, depth 3.
+__device__ __forceinline__ void sort4(uint32_t k[4]) {
+    cmp_swap(k[0], k[1]); cmp_swap(k[2], k[3]);
+    cmp_swap(k[0], k[2]); cmp_swap(k[1], k[3]);
+    cmp_swap(k[1], k[2]);
+}
+// The 7 smallest of the sorted list b[0..7) and the sorted words n[0..4),
+// sorted, in b. The minima of b and the reversed n rise and then fall
+// (bitonic); Batcher's merge of 8 with a lowest word in front (whose
+// comparators do nothing) sorts them: 4 minima and 9 comparators, depth 4.
+__device__ __forceinline__ void merge7(uint32_t b[7], const uint32_t n[4]) {
+    b[3] = min(b[3], n[3]); b[4] = min(b[4], n[2]); b[5] = min(b[5], n[1]); b[6] = min(b[6], n[0]);
+    cmp_swap(b[0], b[4]); cmp_swap(b[1], b[5]); cmp_swap(b[2], b[6]);
+    cmp_swap(b[0], b[2]); cmp_swap(b[3], b[5]); cmp_swap(b[4], b[6]);
+    cmp_swap(b[1], b[2]); cmp_swap(b[3], b[4]); cmp_swap(b[5], b[6]);
+}
+// Inserts w into the sorted list b[0..L): every slot from the old list
+// (min(max(w, b[k - 1]), b[k])), so the chain of a partner is two operations.
+template <int L>
+__device__ __forceinline__ void insert_word(uint32_t* b, uint32_t w) {
+#pragma unroll
+    for (int k = L - 1; k > 0; --k) b[k] = min(max(w, b[k - 1]), b[k]);
+    b[0] = min(b[0], w);
+}
 
-// One partner j of the pair pass: its canonical key |x_j - x_i|^2, the
-// collision flag and Jacobi term (S9, S10) and the downwash term (S10b).
-__device__ __forceinline__ float pair_partner(const Consts& c, const Drone& s, float thr, int tj, const float* sx,
-                                              const float* sv, int nt, bool coll, bool flag_coll, uint32_t& ev,
-                                              float dvs[3], const bool dw, float& dw_az, bool& dw_hit,
-                                              bool& responded) {
+// The K nearest partners of a drone, nearest first: local indices, 8 bits each.
+typedef uint64_t NbrList;
+static_assert(QS_MAX_K <= 8 && QS_MAX_SWARM <= 256, "an NbrList holds QS_MAX_K indices of 8 bits");
+__device__ __forceinline__ int nbr_at(NbrList nb, int k) { return (int)((nb >> (8 * k)) & 0xffu); }
+
+// One partner j of the pair pass that collides or overlaps: the collision flag
+// and Jacobi term (S9, S10) and the downwash term (S10b).
+__device__ __forceinline__ void pair_partner(const Consts& c, const Drone& s, float thr, int tj, const float4* sp,
+                                             const float* sv, int nt, bool coll, bool flag_coll, uint32_t& ev,
+                                             float dvs[3], const bool dw, float& dw_az, bool& dw_hit, bool& responded) {
     float dx, dy, dz;
-    const float key = pair_key(s.x[0], s.x[1], s.x[2], sx[tj], sx[nt + tj], sx[2 * nt + tj], dx, dy, dz);
+    const float4 q = sp[tj];
+    const float key = pair_key(s.x[0], s.x[1], s.x[2], q.x, q.y, q.z, dx, dy, dz);
     // downwash: j overlaps this drone from above (horizontal distance below
     // l_i + l_j, height difference in (0, dw_h))
     if (dw && __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)) < thr && dz > 0.0f && dz < c.dw_h) {
@@ -820,54 +834,177 @@ __device__ __forceinline__ float pair_partner(const Consts& c, const Drone& s, f
             }
         }
     }
-    return key;
+}
+
+template <bool V>
+struct bool_c {
+    static constexpr bool value = V;
+};
+
+// Key and test of partner j at slot-local index j: its word (key bits with the
+// low index bits replaced by j; all ones above them for the drone itself and
+// past the swarm), and whether it collides or overlaps (acc |= ...).
+template <bool DW, bool GUARD>
+__device__ __forceinline__ uint32_t pair_word(const Consts& c, const Drone& s, float thr, const float4& q, int j, int lane,
+                                              int N, uint32_t mask, bool dw, bool& acc) {
+    float dx, dy, dz;
+    const float key = pair_key(s.x[0], s.x[1], s.x[2], q.x, q.y, q.z, dx, dy, dz);
+    const bool out = j == lane || (GUARD && j >= N);
+    const uint32_t kb = out ? 0xffffffffu : __float_as_uint(key);  // all ones: a NaN, below no threshold
+    acc |= __uint_as_float(kb) < thr;
+    if (DW)
+        acc |= dw && !out && __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy)) < thr && dz > 0.0f && dz < c.dw_h;
+    return (kb & ~mask) | (uint32_t)j;
+}
+
+// The words of a swarm of at most M drones (M lanes a slot), sorted when sort.
+// Returns which groups of four partners hold one that collides or overlaps
+// (bit i: partners 4 i to 4 i + 3).
+template <int M, bool DW>
+__device__ __forceinline__ uint32_t pair_words_small(const Consts& c, const Drone& s, float thr, int lane, int N,
+                                                     const float4* sp, bool dw, bool sort, uint32_t b[9]) {
+    bool hit[2] = {false, false};
+    uint32_t w[8];
+#pragma unroll
+    for (int j = 0; j < M; ++j) w[j] = pair_word<DW, true>(c, s, thr, sp[j], j, lane, N, M - 1, dw, hit[j >> 2]);
+    if (sort) {
+        if (M == 2) cmp_swap(w[0], w[1]);
+        if (M == 4) sort4(w);
+        if (M == 8) sort8(w);
+    }
+#pragma unroll
+    for (int k = 0; k < M; ++k) b[k] = w[k];
+    return (hit[0] ? 1u : 0u) | (hit[1] ? 2u : 0u);
+}
+
+// The same for a larger swarm: the L smallest words (L = 0: the tests alone),
+// four partners at a time (a slot has W >= N lanes, a multiple of 4: words past
+// the swarm are all ones).
+template <int L, bool DW>
+__device__ __forceinline__ uint32_t pair_words(const Consts& c, const Drone& s, float thr, int lane, int N,
+                                               const float4* sp, uint32_t mask, bool dw, uint32_t b[9]) {
+    uint32_t hits = 0;
+    const auto four = [&](int j, auto guard) {
+        bool hit = false;
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            w[i] = pair_word<DW, decltype(guard)::value>(c, s, thr, sp[j + i], j + i, lane, N, mask, dw, hit);
+        if constexpr (L == 7) {
+            sort4(w);
+            merge7(b, w);
+        } else if constexpr (L > 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) insert_word<L>(b, w[i]);
+        }
+        if (hit) hits |= 1u << (j >> 2);
+    };
+    int j = 0;
+    for (; j + 4 <= N; j += 4) four(j, bool_c<false>());
+    if (j < N) four(j, bool_c<true>());
+    return hits;
 }
 
 // S9 + S11 for the thread's drone (slot-local index `lane`) against the slot's
-// staged positions / pre-collision velocities (planes of stride nt): collision
-// flag, the Jacobi sum of ((v_j - v_i).n) n over colliding approaching
-// partners (S10), and the sorted neighbour list. Swarms of at most 8 (width
-// classes up to 8, so the test is uniform over a tile) keep every partner's
-// (key, index) word in registers and sort them with a network of 19
-// compare-exchanges; larger swarms insert each partner into the list of the
-// K nearest so far (with K = 6 a list of compile-time length).
+// staged positions (sp: one float4 a drone) and pre-collision velocities
+// (planes of stride nt): collision flag, the Jacobi sum of ((v_j - v_i).n) n
+// over colliding approaching partners (S10), and the list of the keff nearest
+// by (key, index).
+//
+// The selection runs on 32-bit words: the key's bits with the low bits (as
+// many as an index of the slot needs, at most 7) replaced by the partner's
+// index, so a compare-exchange is one minimum and one maximum where the exact
+// (key, index) pair takes a 64-bit compare and four selects. Words order as
+// the exact pairs do unless two keys agree in all their upper bits; the list
+// is one word longer than keff, so any such pair shows as neighbours in it
+// (about 4 drones in 10,000 a step in a swarm of 128), and the exact order is
+// then taken from the keys themselves: of the listed partners, or of all of
+// them when the last listed one is in doubt. Collisions and overlaps are rare:
+// the scan only notes the groups of four partners that hold one, and those are
+// then taken again, in order.
+//
+// Bound by the ALU pipe (minima, maxima, selects) and, with one or two warps a
+// scheduler, by the chain of a partner's insertion; against 64-bit words, one
+// partner at a time: 256 swarms of 128, 16 steps 405 -> 203 us (75 -> 30
+// instructions a partner), 4096 uneven swarms, 32 steps 625 -> 358 us, 2048
+// swarms of 8, 64 steps 242 -> 216 us.
+template <bool DW>
 __device__ __forceinline__ bool pair_scan(const Consts& c, const Drone& s, float thr, int lane, int N, int sbase,
-                                          const float* sx, const float* sv, int nt, int keff, bool coll, bool flag_coll,
-                                          uint32_t& ev, uint64_t best[QS_MAX_K], float dvs[3], const bool dw,
-                                          float& dw_az, bool& dw_hit) {
-    bool responded = false;
-    if (N <= 8) {
-        uint64_t kk[8];
+                                          const float4* spos, const float* sv, int nt, int keff, bool coll, bool flag_coll,
+                                          uint32_t& ev, NbrList& nbrs, float dvs[3], const bool dw, float& dw_az,
+                                          bool& dw_hit) {
+    const float4* sp = spos + sbase;
+    uint32_t b[9];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            kk[j] = ~0ull;
-            if (j < N && j != lane) {
-                const float key = pair_partner(c, s, thr, sbase + j, sx, sv, nt, coll, flag_coll, ev, dvs, dw, dw_az,
-                                               dw_hit, responded);
-                kk[j] = ((uint64_t)__float_as_uint(key) << 32) | (uint32_t)j;
+    for (int k = 0; k < 9; ++k) b[k] = 0xffffffffu;
+    uint32_t mask;
+    uint32_t hits;  // groups of four partners
+    if (N <= 2) {
+        mask = 1u;
+        hits = pair_words_small<2, DW>(c, s, thr, lane, N, sp, dw, keff > 0, b);
+    } else if (N <= 4) {
+        mask = 3u;
+        hits = pair_words_small<4, DW>(c, s, thr, lane, N, sp, dw, keff > 0, b);
+    } else if (N <= 8) {
+        mask = 7u;
+        hits = pair_words_small<8, DW>(c, s, thr, lane, N, sp, dw, keff > 0, b);
+    } else {
+        mask = N <= 16 ? 15u : N <= 32 ? 31u : N <= 64 ? 63u : 127u;
+        if (keff == 0)
+            hits = pair_words<0, DW>(c, s, thr, lane, N, sp, mask, dw, b);
+        else if (keff <= 6)
+            hits = pair_words<7, DW>(c, s, thr, lane, N, sp, mask, dw, b);
+        else
+            hits = pair_words<9, DW>(c, s, thr, lane, N, sp, mask, dw, b);
+    }
+    bool responded = false;
+    if (!flag_coll && !dw) hits = 0;
+    while (hits) {
+        const int j0 = 4 * (__ffs(hits) - 1), j1 = min(j0 + 4, N);
+        hits &= hits - 1;
+        for (int j = j0; j < j1; ++j)
+            if (j != lane)
+                pair_partner(c, s, thr, sbase + j, spos, sv, nt, coll, flag_coll, ev, dvs, dw, dw_az, dw_hit, responded);
+    }
+    nbrs = 0;
+    if (keff == 0) return responded;
+    bool doubt = false, last = false;
+#pragma unroll
+    for (int k = 0; k < QS_MAX_K; ++k) {
+        if (k < keff) {
+            const bool same = ((b[k] ^ b[k + 1]) & ~mask) == 0u;
+            doubt |= same;
+            last = same;
+            nbrs |= (NbrList)(b[k] & mask) << (8 * k);
+        }
+    }
+    if (doubt) {
+        uint64_t best[QS_MAX_K];  // (key, index) words
+        const auto word = [&](int j) {
+            float dx, dy, dz;
+            const float4 q = sp[j];
+            return (uint64_t)__float_as_uint(pair_key(s.x[0], s.x[1], s.x[2], q.x, q.y, q.z, dx, dy, dz)) << 32 | (uint32_t)j;
+        };
+        if (N <= 8) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) best[j] = j < N && j != lane ? word(j) : ~0ull;
+            sort8(best);
+        } else {
+#pragma unroll
+            for (int k = 0; k < QS_MAX_K; ++k) best[k] = ~0ull;
+            const int n = last ? N : keff;
+            for (int t = 0; t < n; ++t) {
+                const int j = last ? t : nbr_at(nbrs, t);
+                if (j == lane) continue;
+                uint64_t w = word(j);
+#pragma unroll
+                for (int k = 0; k < QS_MAX_K; ++k) cmp_swap(best[k], w);
             }
         }
-        if (keff > 0) {
-            sort8(kk);
+        nbrs = 0;
 #pragma unroll
-            for (int k = 0; k < QS_MAX_K; ++k) best[k] = k < keff ? kk[k] : ~0ull;
-        }
-        return responded;
-    }
-    if (keff == 6) {  // the paper's K (N > 8 here, so keff = K): the list length fixed
-        for (int j = 0; j < N; ++j) {
-            if (j == lane) continue;
-            const float key = pair_partner(c, s, thr, sbase + j, sx, sv, nt, coll, flag_coll, ev, dvs, dw, dw_az,
-                                           dw_hit, responded);
-            topk_insert_n<6>(best, ((uint64_t)__float_as_uint(key) << 32) | (uint32_t)j);
-        }
-        return responded;
-    }
-    for (int j = 0; j < N; ++j) {
-        if (j == lane) continue;
-        const float key = pair_partner(c, s, thr, sbase + j, sx, sv, nt, coll, flag_coll, ev, dvs, dw, dw_az, dw_hit,
-                                       responded);
-        if (keff > 0) topk_insert(best, keff, ((uint64_t)__float_as_uint(key) << 32) | (uint32_t)j);
+        for (int k = 0; k < QS_MAX_K; ++k)
+            if (k < keff) nbrs |= (NbrList)(best[k] & 0xffu) << (8 * k);
     }
     return responded;
 }

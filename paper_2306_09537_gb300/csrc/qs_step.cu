@@ -13,7 +13,7 @@
 // env. For W > 1 the slot exchanges positions and velocities through shared
 // memory for the O(N^2) pair pass (collisions, Sec. III-B) and the K-nearest
 // neighbour selection (Sec. II-B, III-C), which each thread keeps as a sorted
-// register list of 64-bit keys (binary32 distance bits << 32 | index).
+// register list of 32-bit words (pair_scan).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -24,9 +24,12 @@
 namespace qsk {
 
 constexpr int MAX_BLOCK = 256;
-// dynamic shared memory of the step and rollout kernels, per thread: staged
-// position (3) and velocity (3) of the pair pass, swap key (1)
-constexpr int SMEM_PLANES = 7;
+// dynamic shared memory of the step and rollout kernels, floats per thread:
+// staged position (4: one 16-byte load a partner) and velocity (3) of the pair
+// pass, swap key (1). The rollout stages by step parity in two such sets: a
+// slot wider than a warp would otherwise stage step t + 1 over what its slower
+// warps still read for step t's neighbour rows.
+constexpr int SMEM_PLANES = 8;
 
 // The step kernels come in two instances: EXT = true carries the training
 // scenarios (per-drone goals), the downwash term and the smooth contacts,
@@ -103,9 +106,10 @@ __device__ __forceinline__ void apply_downwash(const Consts& c, Drone& s, uint32
 }
 
 // S13 reward of one drone (Sec. III-E): weighted state terms, event indicators
-// and the proximity term over its neighbours (keys = squared distances).
+// and the proximity term over its keff neighbours (pos(k): position of the k-th).
+template <class Pos>
 __device__ __forceinline__ float compute_reward(const Consts& c, const Drone& s, float prox, const float g[3],
-                                                const float fh[4], uint32_t ev, const uint64_t best[QS_MAX_K], int keff) {
+                                                const float fh[4], uint32_t ev, int keff, const Pos& pos) {
     // explicit roundings: the same bits from every kernel that computes it
     const float dgx = __fsub_rn(s.x[0], g[0]), dgy = __fsub_rn(s.x[1], g[1]), dgz = __fsub_rn(s.x[2], g[2]);
     float r = __fmul_rn(c.w[QS_W_POS], sqrt_approx(dot3(dgx, dgy, dgz, dgx, dgy, dgz)));
@@ -131,7 +135,9 @@ __device__ __forceinline__ float compute_reward(const Consts& c, const Drone& s,
 #pragma unroll
         for (int k = 0; k < QS_MAX_K; ++k) {
             if (k < keff) {
-                const float key = __uint_as_float((uint32_t)(best[k] >> 32));
+                const float3 q = pos(k);
+                float dx, dy, dz;
+                const float key = pair_key(s.x[0], s.x[1], s.x[2], q.x, q.y, q.z, dx, dy, dz);
                 near = __fadd_rn(near, fmaxf(__fmaf_rn(-sqrt_approx(key), inv_prox, 1.0f), 0.0f));
             }
         }
@@ -187,7 +193,7 @@ __device__ __forceinline__ void end_step(const Consts& c, const Dev& dv, Drone& 
 // uniform over the CTA; a compile-time W folds away after inlining.
 template <bool EXT>
 __device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, uint32_t& ev_out,
-                                          float* sx, float* sv, const bool act, const int lane, const int N,
+                                          float4* sp, float* sv, const bool act, const int lane, const int N,
                                           const int sbase, const int e, const int d, const float4 a,
                                           float* __restrict__ obs, float* __restrict__ rew, uint8_t* __restrict__ done,
                                           const int observe_only, GoalCache& gc) {
@@ -218,13 +224,9 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         const float u[4] = {sqrt_approx(fh[0]), sqrt_approx(fh[1]), sqrt_approx(fh[2]), sqrt_approx(fh[3])};
         for (int sub = 0; sub < c.substeps; ++sub) {
             float pacc[3] = {0.f, 0.f, 0.f};
-            if (act) {
-                sx[threadIdx.x] = s.x[0];
-                sx[nt + threadIdx.x] = s.x[1];
-                sx[2 * nt + threadIdx.x] = s.x[2];
-            }
+            if (act) sp[threadIdx.x] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
             __syncthreads();
-            if (act && N > 1) pair_acc(c, s.x, sx, nt, sbase, lane, N, er.p.arm, pacc);
+            if (act && N > 1) pair_acc(c, s.x, sp, sbase, lane, N, er.p.arm, pacc);
             __syncthreads();
             if (act) ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, tick, d, sub, pacc);
         }
@@ -239,14 +241,10 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
     }
 
     // ---- pair pass: collisions (S9, S10) and K nearest neighbours (S11)
-    uint64_t best[QS_MAX_K];
-#pragma unroll
-    for (int k = 0; k < QS_MAX_K; ++k) best[k] = ~0ull;
+    NbrList nbrs = 0;
     if (W > 1) {
         if (act) {
-            sx[threadIdx.x] = s.x[0];
-            sx[nt + threadIdx.x] = s.x[1];
-            sx[2 * nt + threadIdx.x] = s.x[2];
+            sp[threadIdx.x] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
             sv[threadIdx.x] = s.v[0];
             sv[nt + threadIdx.x] = s.v[1];
             sv[2 * nt + threadIdx.x] = s.v[2];
@@ -258,8 +256,8 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         if (act && N > 1) {
             const bool coll = (c.flags & QS_F_COLLISIONS) && !(EXT && (c.flags & QS_F_SMOOTH)) && !observe_only;
             const bool flag_coll = (c.flags & QS_F_COLLISIONS) && !observe_only;
-            responded = pair_scan(c, s, er.p.thr, lane, N, sbase, sx, sv, nt, keff, coll, flag_coll, ev, best, dvs,
-                                  dw && !observe_only, dw_az, dw_hit);
+            responded = pair_scan<EXT>(c, s, er.p.thr, lane, N, sbase, sp, sv, nt, keff, coll, flag_coll, ev, nbrs, dvs,
+                                       dw && !observe_only, dw_az, dw_hit);
         }
         if (responded) apply_response(c, s, tick, d, dvs);
         if (dw && dw_hit && !observe_only) apply_downwash(c, s, tick, d, dw_az);
@@ -311,9 +309,10 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
             if (k >= K) break;
             float2* on = o2 + 9 + 3 * k;
             if (W > 1 && k < keff) {
-                const int tj = sbase + (int)(best[k] & 0xffffffffu);
-                on[0] = make_float2(sx[tj] - s.x[0], sx[nt + tj] - s.x[1]);
-                on[1] = make_float2(sx[2 * nt + tj] - s.x[2], sv[tj] - s.v[0]);
+                const int tj = sbase + nbr_at(nbrs, k);
+                const float4 q = sp[tj];
+                on[0] = make_float2(q.x - s.x[0], q.y - s.x[1]);
+                on[1] = make_float2(q.z - s.x[2], sv[tj] - s.v[0]);
                 on[2] = make_float2(sv[nt + tj] - s.v[1], sv[2 * nt + tj] - s.v[2]);
             } else {
                 on[0] = make_float2(0.f, 0.f);
@@ -327,12 +326,16 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
     if ((c.flags & QS_F_RECORD_KNN) && dv.knn) {
 #pragma unroll
         for (int k = 0; k < QS_MAX_K; ++k)
-            if (k < K) dv.knn[(size_t)k * dv.D + d] = k < keff ? (int16_t)(best[k] & 0xffffu) : (int16_t)-1;
+            if (k < K) dv.knn[(size_t)k * dv.D + d] = (W > 1 && k < keff) ? (int16_t)nbr_at(nbrs, k) : (int16_t)-1;
     }
     ev_out = ev;
 
     // ---- S13 reward and done
-    if (rew) rew[d] = compute_reward(c, s, er.p.prox, gl, fh, ev, best, W > 1 ? keff : 0);
+    if (rew)
+        rew[d] = compute_reward(c, s, er.p.prox, gl, fh, ev, W > 1 ? keff : 0, [&](int k) {
+            const float4 q = sp[sbase + nbr_at(nbrs, k)];
+            return make_float3(q.x, q.y, q.z);
+        });
     end_step<EXT>(c, dv, s, er, fh, lane, e, d, done);
     if (scn && er.ep == 0) gc.until = -1;  // an auto-reset drew a new record
 }
@@ -362,7 +365,7 @@ __device__ __forceinline__ SlotMap map_slot(const Dev& dv, const Tile& tile, con
 template <int W, bool EXT>
 __global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                     const int* __restrict__ perm, const StepIO io, const int observe_only) {
-    extern __shared__ float sm[];
+    extern __shared__ float4 sm[];
     const SlotMap m = map_slot(dv, tile_at(dv, tiles, blockIdx.x, blockDim.x), perm, W);
     Drone s;
     EnvRegs er;
@@ -374,7 +377,7 @@ __global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Cons
     const float4 a = (m.act && !observe_only) ? __ldg(reinterpret_cast<const float4*>(io.act) + m.d)
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
     GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
-    step_body<EXT>(W, c, dv, s, er, ev, sm, sm + 3 * blockDim.x, m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
+    step_body<EXT>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
               io.rew, io.done, observe_only, gc);
     if (!m.act || observe_only) return;
     dv.ev[m.d] = ev;
@@ -387,7 +390,7 @@ __global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Cons
 // neighbour or staging code).
 template <bool EXT, bool W1>
 __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, const Tile& tile, const int* __restrict__ perm,
-                                             float* sm, const RolloutIO& io, int t0, int nsteps) {
+                                             float4* sm, const RolloutIO& io, int t0, int nsteps) {
     const int W = W1 ? 1 : tile.W;
     const SlotMap m = map_slot(dv, tile, perm, W);
     Drone s;
@@ -406,7 +409,8 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
     for (int t = t0; t < t0 + nsteps; ++t) {
         const float4 a = a_next;
         if (m.act && t + 1 < t0 + nsteps) a_next = __ldg(act4 + (size_t)(t + 1) * D);
-        step_body<EXT>(W, c, dv, s, er, ev, sm, sm + 3 * blockDim.x, m.act, m.lane, m.N, m.sbase, m.e, m.d, a,
+        float4* sp = sm + ((t - t0) & 1) * (SMEM_PLANES / 4) * blockDim.x;
+        step_body<EXT>(W, c, dv, s, er, ev, sp, reinterpret_cast<float*>(sp + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a,
                        io.obs ? io.obs + (size_t)t * D * c.obs_dim : nullptr, io.rew ? io.rew + (size_t)t * D : nullptr,
                        io.done ? io.done + (size_t)t * E : nullptr, 0, gc);
     }
@@ -429,7 +433,7 @@ __global__ void __launch_bounds__(MAX_BLOCK, 2) k_rollout(const Consts c, const 
                                                        const int n_tiles, const int* __restrict__ perm,
                                                        int* __restrict__ counter, const RolloutIO io, const int t0,
                                                        const int nsteps) {
-    extern __shared__ float sm[];
+    extern __shared__ float4 sm[];
     __shared__ int s_next;
     for (;;) {
         if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
@@ -468,7 +472,7 @@ struct WsShared {
     int keff[2][32 * P];
     float rin[2][9][32 * P];          // reward inputs: command f^ (4), previous command (4), proximity radius
     uint32_t ev[2][32 * P];           // event bits
-    float sx[3][32 * P];              // pair-pass staging: positions
+    float4 sp[32 * P];                // pair-pass staging: positions
     float sv[3][32 * P];              //                    velocities
     uint32_t key[32 * P];             // swap keys
     float rows[32 * P * WS_OBS_MAX];
@@ -624,13 +628,9 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
     if (spair) {
         for (int sub = 0; sub < c.substeps; ++sub) {
             float pacc[3] = {0.f, 0.f, 0.f};
-            if (act) {
-                sh.sx[0][L] = s.x[0];
-                sh.sx[1][L] = s.x[1];
-                sh.sx[2][L] = s.x[2];
-            }
+            if (act) sh.sp[L] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
             side_sync<P>(1);
-            if (act && N > 1) pair_acc(c, s.x, &sh.sx[0][0], 32 * P, sbase, lane, N, er.p.arm, pacc);
+            if (act && N > 1) pair_acc(c, s.x, sh.sp, sbase, lane, N, er.p.arm, pacc);
             side_sync<P>(1);
             if (act) {
                 if (mnoise && sub < nahead) {
@@ -655,14 +655,10 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         }
     }
     const int keff = min(K, N - 1);
-    uint64_t best[QS_MAX_K];
-#pragma unroll
-    for (int k = 0; k < QS_MAX_K; ++k) best[k] = ~0ull;
+    NbrList nbrs = 0;
     if (W > 1) {
         if (act) {
-            sh.sx[0][L] = s.x[0];
-            sh.sx[1][L] = s.x[1];
-            sh.sx[2][L] = s.x[2];
+            sh.sp[L] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
             sh.sv[0][L] = s.v[0];
             sh.sv[1][L] = s.v[1];
             sh.sv[2][L] = s.v[2];
@@ -674,8 +670,8 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         if (act && N > 1) {
             const bool coll = (c.flags & QS_F_COLLISIONS) && !(EXT && (c.flags & QS_F_SMOOTH));
             const bool flag_coll = (c.flags & QS_F_COLLISIONS) != 0;
-            responded = pair_scan(c, s, er.p.thr, lane, N, sbase, &sh.sx[0][0], &sh.sv[0][0], 32 * P, keff, coll,
-                                  flag_coll, ev, best, dvs, dw, dw_az, dw_hit);
+            responded = pair_scan<EXT>(c, s, er.p.thr, lane, N, sbase, sh.sp, &sh.sv[0][0], 32 * P, keff, coll, flag_coll,
+                                       ev, nbrs, dvs, dw, dw_az, dw_hit);
         }
         if (responded) apply_response(c, s, er.tick, d, dvs);
         if (dw && dw_hit) apply_downwash(c, s, er.tick, d, dw_az);
@@ -716,7 +712,7 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         sh.keff[b][L] = W > 1 ? keff : 0;
 #pragma unroll
         for (int k = 0; k < QS_MAX_K; ++k)
-            if (k < keff) sh.nb[b][k][L] = sbase + (int)(best[k] & 0xffffffffu);
+            if (k < keff) sh.nb[b][k][L] = sbase + nbr_at(nbrs, k);
         if (DEFER) {  // the noise side computes the reward from these
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -732,17 +728,20 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
     if ((c.flags & QS_F_RECORD_KNN) && dv.knn) {
 #pragma unroll
         for (int k = 0; k < QS_MAX_K; ++k)
-            if (k < K) dv.knn[(size_t)k * dv.D + d] = (W > 1 && k < keff) ? (int16_t)(best[k] & 0xffffu) : (int16_t)-1;
+            if (k < K) dv.knn[(size_t)k * dv.D + d] = (W > 1 && k < keff) ? (int16_t)nbr_at(nbrs, k) : (int16_t)-1;
     }
-    if (!DEFER && rew) rew[d] = compute_reward(c, s, er.p.prox, gl, fh, ev, best, W > 1 ? keff : 0);
+    if (!DEFER && rew)
+        rew[d] = compute_reward(c, s, er.p.prox, gl, fh, ev, W > 1 ? keff : 0, [&](int k) {
+            const float4 q = sh.sp[sbase + nbr_at(nbrs, k)];
+            return make_float3(q.x, q.y, q.z);
+        });
     end_step<EXT>(c, dv, s, er, fh, lane, e, d, done);
     if (EXT && er.ep == 0) gc.until = -1;  // an auto-reset drew a new record
     ev_out = ev;
 }
 
 // Noise side: the reward of the step published in buffer b (the same
-// compute_reward as the dynamics side, on the published post-step state; the
-// neighbour keys recomputed with the canonical pair key on the same positions).
+// compute_reward as the dynamics side, on the published post-step state).
 template <int P>
 __device__ __forceinline__ void ws_reward(const Consts& c, WsShared<P>& sh, const WsMap& m, int b,
                                           float* __restrict__ rew) {
@@ -761,19 +760,10 @@ __device__ __forceinline__ void ws_reward(const Consts& c, WsShared<P>& sh, cons
         s.fp[r] = sh.rin[b][4 + r][L];
     }
     const float g[3] = {sh.g[b][0][L], sh.g[b][1][L], sh.g[b][2][L]};
-    const int keff = sh.keff[b][L];
-    uint64_t best[QS_MAX_K];
-#pragma unroll
-    for (int k = 0; k < QS_MAX_K; ++k) {
-        best[k] = ~0ull;
-        if (k < keff) {
-            const int j = sh.nb[b][k][L];
-            float dx, dy, dz;
-            const float key = pair_key(s.x[0], s.x[1], s.x[2], sh.st[b][0][j], sh.st[b][1][j], sh.st[b][2][j], dx, dy, dz);
-            best[k] = (uint64_t)__float_as_uint(key) << 32;
-        }
-    }
-    rew[m.d] = compute_reward(c, s, sh.rin[b][8][L], g, fh, sh.ev[b][L], best, keff);
+    rew[m.d] = compute_reward(c, s, sh.rin[b][8][L], g, fh, sh.ev[b][L], sh.keff[b][L], [&](int k) {
+        const int j = sh.nb[b][k][L];
+        return make_float3(sh.st[b][0][j], sh.st[b][1][j], sh.st[b][2][j]);
+    });
 }
 
 template <bool EXT>
@@ -1140,7 +1130,7 @@ int rollout_grid(int block, bool ext, bool single) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, rollout_kernel(ext, single), block,
-                                                  sizeof(float) * SMEM_PLANES * block);
+                                                  sizeof(float) * 2 * SMEM_PLANES * block);
     return (occ > 0 ? occ : 1) * n_sm;
 }
 
@@ -1169,7 +1159,7 @@ cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, in
                            cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    const size_t smem = sizeof(float) * SMEM_PLANES * block;
+    const size_t smem = sizeof(float) * 2 * SMEM_PLANES * block;
     const int g = grid > 0 ? grid : n_tiles;
     const int grid_n = g < n_tiles ? g : n_tiles;
     if (extended(c))
