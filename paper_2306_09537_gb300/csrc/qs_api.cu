@@ -324,7 +324,7 @@ qs_status upload_tiles(qs_env* h) {
     h->d_wtiles = h->d_tiles + n0 + n1 + n2;
     h->n_wtiles = (int)wtiles.size();
     h->single_drone = maxW == 1;
-    h->rollout_grid = rollout_grid(rblock, extended_instance(h->c), h->single_drone);
+    h->rollout_grid = rollout_grid(h->c, rblock, h->single_drone);
     return QS_OK;
 }
 
@@ -344,12 +344,22 @@ qs_status enqueue_rollout(qs_env* h, int T, const RolloutIO& io) {
 }
 
 
+// Whether p is memory of a device (not page-locked, managed or plain host memory).
+bool device_memory(const void* p) {
+    cudaPointerAttributes a;
+    if (!p || cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice;
+}
+
 // One control step of every env. A handle with several width classes steps
 // them all in one launch of the rollout kernels with T = 1 (the same bits as
 // the per-class kernels; measured on GB300 with sizes 1..64: 4096 envs 90.8
 // -> 35.5 us, 65,536 envs 271 -> 207 us); one class keeps its per-call kernel.
 qs_status do_step(qs_env* h, const float* act, float* obs, float* rew, uint8_t* done) {
-    if (h->plan.size() > 1) return enqueue_rollout(h, 1, RolloutIO{act, obs, rew, done});
+    if (h->plan.size() > 1) return enqueue_rollout(h, 1, RolloutIO{act, obs, rew, done, device_memory(obs)});
     StepIO io{act, obs, rew, done};
     for (const ClassPlan& cp : h->plan) {
         cudaError_t e = launch_step(h->c, h->dv, cp, h->d_tiles, h->d_perm, io, 0, h->stream);
@@ -760,11 +770,11 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
     if (!actions_dev || !aligned(actions_dev, 16)) return fail(h, QS_ERR_ARG, "qs_rollout: actions_dev NULL or misaligned");
     if (obs_dev && !aligned(obs_dev, 8)) return fail(h, QS_ERR_ARG, "qs_rollout: obs_dev must be 8-byte aligned");
     DeviceGuard g(h->device);
-    const RolloutIO io{actions_dev, obs_dev, reward_dev, done_dev};
     // Graph replay: the launches of one (T, buffers, shape) are captured once
     // and replayed; any change of buffers or shape re-captures. The legacy
     // default stream cannot be captured, so it launches directly.
-    if (!h->use_graph || h->stream == nullptr) return enqueue_rollout(h, T, io);
+    if (!h->use_graph || h->stream == nullptr)
+        return enqueue_rollout(h, T, RolloutIO{actions_dev, obs_dev, reward_dev, done_dev, device_memory(obs_dev)});
     const auto& k = h->graph_key;
     if (h->graph && k.T == T && k.fuse == h->rollout_fuse && k.block == h->rollout_block && k.a == actions_dev &&
         k.o == obs_dev && k.r == reward_dev && k.d == done_dev) {
@@ -772,6 +782,7 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
         return e == cudaSuccess ? QS_OK : cuda_fail(h, e, "rollout graph launch");
     }
     drop_graph(h);
+    const RolloutIO io{actions_dev, obs_dev, reward_dev, done_dev, device_memory(obs_dev)};
     cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(h, e, "rollout capture begin");
     qs_status s = enqueue_rollout(h, T, io);

@@ -122,6 +122,7 @@ struct RolloutIO {
     float* obs;        // [T][D][obs_dim]
     float* rew;        // [T][D]
     uint8_t* done;     // [T][E]
+    bool bulk;         // obs is device memory (rows may leave by bulk asynchronous copies)
 };
 
 // kernels (qs_step.cu)
@@ -163,9 +164,8 @@ int serve_resident_ctas(const Consts& c, int P);
 // resident at once.
 int rollout_ws_resident_ctas(const Consts& c, int P);
 // CTAs of `block` threads the device keeps resident at once for the k_rollout
-// instance launch_rollout picks (extended: extended_instance(); single: one
-// drone per env).
-int rollout_grid(int block, bool extended, bool single);
+// instance launch_rollout picks (single: one drone per env).
+int rollout_grid(const Consts& c, int block, bool single);
 
 // differentiable rollout (qs_adjoint.cu)
 size_t diff_workspace_bytes(int D, int T, int C, int substeps);

@@ -30,6 +30,11 @@ constexpr int MAX_BLOCK = 256;
 // slot wider than a warp would otherwise stage step t + 1 over what its slower
 // warps still read for step t's neighbour rows.
 constexpr int SMEM_PLANES = 8;
+// the rollout's observation rows in shared memory, floats per thread: a row and
+// the padding of its block (RowMap)
+constexpr int ROW_PAD = 6;
+// and the most the kernels ask for
+constexpr int STEP_SMEM_MAX = (int)sizeof(float) * MAX_BLOCK * (2 * SMEM_PLANES + 18 + 6 * QS_MAX_K + ROW_PAD);
 
 // The step kernels come in two instances: EXT = true carries the training
 // scenarios (per-drone goals), the downwash term and the smooth contacts,
@@ -187,16 +192,92 @@ __device__ __forceinline__ void end_step(const Consts& c, const Dev& dv, Drone& 
     if (!finite_state(s)) atomicOr(dv.status, 1);
 }
 
+// Observation rows of a warp's drones on their way to memory. A row is od
+// floats and a lane owns one, so rows written lane by lane put every store of a
+// warp into 32 distinct sectors (K = 6: 27 stores of 8 bytes, 864 sectors for
+// 216), and the warp waits for them before it may overwrite the registers they
+// read. The rollout puts the rows together in shared memory instead and hands
+// each block of consecutive rows to one bulk asynchronous copy, which runs
+// while the warp computes the next step. The drones of a warp usually follow
+// one another and form one block; the envs of a mixed handle's tile need not,
+// and then each slot is a block. A bulk copy moves 16-byte units between
+// addresses of the same offset: a block starts at its destination's offset
+// within 16 bytes, and the 8 bytes before or after the units are stored apart.
+struct RowMap {
+    int d0, n;   // first drone and rows of the lane's block
+    int off;     // the block's floats in the warp's buffer start here (a multiple of 4)
+    int rank;    // row of this lane's drone in it
+    bool lead;   // this lane copies the block
+};
+
+__device__ __forceinline__ RowMap map_rows(bool act, int d, int W, int od) {
+    RowMap r;
+    const uint32_t am = __ballot_sync(0xffffffffu, act);
+    const int ln = threadIdx.x & 31, rank = __popc(am & ((1u << ln) - 1u)), lead = max(__ffs(am) - 1, 0);
+    const int f0 = __shfl_sync(0xffffffffu, d - rank, lead);
+    const bool one = __all_sync(0xffffffffu, !act || d - rank == f0);
+    if (one) {
+        r = RowMap{f0, __popc(am), 0, rank, act && ln == lead};
+    } else {  // slots of one warp: W <= 16
+        const int slot = ln / W, l0 = slot * W;
+        r = RowMap{d - (ln - l0), __popc(am >> l0 & ((1u << W) - 1u)), slot * (((W * od + 3) & ~3) + 4), ln - l0,
+                   act && ln == l0};
+    }
+    return r;
+}
+
+// Floats from the block's start to its first row: the offset of the destination within 16 bytes.
+__device__ __forceinline__ int row_shift(const RowMap& r, const float* obs, int od) {
+    return (int)((uintptr_t)(obs + (size_t)r.d0 * od) >> 2) & 3;
+}
+
+// Before the rows of another step are written: the copies have read the last one's.
+__device__ __forceinline__ void rows_free(const RowMap& r) {
+    if (r.lead) asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+    __syncwarp();
+}
+
+// Starts the copies of the warp's blocks (every lane calls it), or without
+// bulk (a destination in host memory) stores each lane's row.
+__device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, float* __restrict__ obs, int od, bool act,
+                                          bool bulk) {
+    float* dst = obs + (size_t)r.d0 * od;
+    const int sh = row_shift(r, obs, od);
+    const float* src = rows + r.off + sh;
+    if (!bulk) {
+        const float2* s2 = reinterpret_cast<const float2*>(src + r.rank * od);
+        float2* d2 = reinterpret_cast<float2*>(dst + (size_t)r.rank * od);
+        if (act)
+            for (int i = 0; i < od / 2; ++i) d2[i] = s2[i];
+        return;
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+    if (r.lead) {
+        const int n = r.n * od - sh, m = n & ~3;  // floats past the 8 bytes before the units
+        if (sh) *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(src);
+        if (n & 2) *reinterpret_cast<float2*>(dst + sh + m) = *reinterpret_cast<const float2*>(src + sh + m);
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(dst + sh),
+                     "r"((uint32_t)__cvta_generic_to_shared(src + sh)), "r"(4 * m)
+                     : "memory");
+    }
+}
+
 // One control step of the slot's drones. All threads of the CTA call it (the
 // pair pass synchronises the CTA); `act` marks threads that carry a drone.
 // Outputs for this step: obs/rew rows of drone d, done[e] (lane 0). W is
 // uniform over the CTA; a compile-time W folds away after inlining.
-template <bool EXT>
+// ROWS: the observation rows go through shared memory (the rollout), else each
+// lane stores its own. Swarm rollouts take the former (4096 uneven swarms, 32
+// steps, 358 -> 299 us; 256 x 128, 16 steps, 203 -> 183 us); single drones keep
+// their 9 stores: addressing the block costs 95 instructions of 1,100 a step,
+// more than the stores' waits (1,048,576 drones, 32 steps: 1696 against 1834 us).
+template <bool EXT, bool ROWS>
 __device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, uint32_t& ev_out,
                                           float4* sp, float* sv, const bool act, const int lane, const int N,
                                           const int sbase, const int e, const int d, const float4 a,
                                           float* __restrict__ obs, float* __restrict__ rew, uint8_t* __restrict__ done,
-                                          const int observe_only, GoalCache& gc) {
+                                          const int observe_only, GoalCache& gc, const RowMap& rm, float* rows, const bool bulk) {
     const int nt = blockDim.x;
     const int K = c.K;
     const int keff = min(K, N - 1);
@@ -274,11 +355,11 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         }
         __syncthreads();
     }
-    if (!act) return;
+    if (!ROWS && !act) return;
 
     // ---- the drone's goal at the end of the step (Sec. III-D scenarios)
     float gl[3] = {er.g0, er.g1, er.g2};
-    if (scn) {
+    if (scn && act) {
         if (goal_cached(gc, tau)) {
             gl[0] = gc.g[0];
             gl[1] = gc.g[1];
@@ -291,10 +372,12 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
     }
 
     // ---- S12 observation
-    if (obs) {
+    if (ROWS && obs) rows_free(rm);
+    if (obs && act) {
         float ex[3] = {0.f, 0.f, 0.f}, evv[3] = {0.f, 0.f, 0.f}, ew[3] = {0.f, 0.f, 0.f};
         if (c.flags & QS_F_OBS_NOISE) obs_noise(c, tick, d, observe_only ? 1u : 0u, ex, evv, ew);
-        float2* o2 = reinterpret_cast<float2*>(obs + (size_t)d * c.obs_dim);
+        float2* o2 = reinterpret_cast<float2*>(ROWS ? rows + rm.off + row_shift(rm, obs, c.obs_dim) + rm.rank * c.obs_dim
+                                                    : obs + (size_t)d * c.obs_dim);
         o2[0] = make_float2(s.x[0] - gl[0] + ex[0], s.x[1] - gl[1] + ex[1]);
         o2[1] = make_float2(s.x[2] - gl[2] + ex[2], s.v[0] + evv[0]);
         o2[2] = make_float2(s.v[1] + evv[1], s.v[2] + evv[2]);
@@ -321,7 +404,8 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
             }
         }
     }
-    if (observe_only) return;
+    if (ROWS && obs) send_rows(rm, rows, obs, c.obs_dim, act, bulk);
+    if (!act || observe_only) return;
 
     if ((c.flags & QS_F_RECORD_KNN) && dv.knn) {
 #pragma unroll
@@ -377,8 +461,8 @@ __global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Cons
     const float4 a = (m.act && !observe_only) ? __ldg(reinterpret_cast<const float4*>(io.act) + m.d)
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
     GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
-    step_body<EXT>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
-              io.rew, io.done, observe_only, gc);
+    step_body<EXT, false>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
+              io.rew, io.done, observe_only, gc, RowMap(), nullptr, false);
     if (!m.act || observe_only) return;
     dv.ev[m.d] = ev;
     store_drone(s, dv.st, dv.D, m.d);
@@ -406,14 +490,17 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
     // HBM latency leaves each step's dependent chain
     float4 a_next = m.act ? __ldg(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
     GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
+    const RowMap rm = W1 ? RowMap() : map_rows(m.act, m.d, W, c.obs_dim);
+    float* rows = reinterpret_cast<float*>(sm + 2 * SMEM_PLANES / 4 * blockDim.x) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
     for (int t = t0; t < t0 + nsteps; ++t) {
         const float4 a = a_next;
         if (m.act && t + 1 < t0 + nsteps) a_next = __ldg(act4 + (size_t)(t + 1) * D);
         float4* sp = sm + ((t - t0) & 1) * (SMEM_PLANES / 4) * blockDim.x;
-        step_body<EXT>(W, c, dv, s, er, ev, sp, reinterpret_cast<float*>(sp + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a,
+        step_body<EXT, !W1>(W, c, dv, s, er, ev, sp, reinterpret_cast<float*>(sp + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a,
                        io.obs ? io.obs + (size_t)t * D * c.obs_dim : nullptr, io.rew ? io.rew + (size_t)t * D : nullptr,
-                       io.done ? io.done + (size_t)t * E : nullptr, 0, gc);
+                       io.done ? io.done + (size_t)t * E : nullptr, 0, gc, rm, rows, io.bulk);
     }
+    if (!W1 && rm.lead) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (m.act) {
         dv.ev[m.d] = ev;
         store_drone(s, dv.st, dv.D, m.d);
@@ -1125,12 +1212,27 @@ const void* rollout_kernel(bool ext, bool single) {
     return single ? (const void*)k_rollout<false, true> : (const void*)k_rollout<false, false>;
 }
 
-int rollout_grid(int block, bool ext, bool single) {
+// A rollout kernel whose shared memory passes the 48 KiB every kernel may have (large
+// CTAs with many neighbours) asks for the most any shape needs, so that no
+// handle's call lowers another's.
+cudaError_t allow_smem(const void* fn, size_t smem) {
+    return smem <= 48u << 10 ? cudaSuccess : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM_MAX);
+}
+
+// Its dynamic shared memory: two sets of staging planes and the CTA's
+// observation rows (none for single drones).
+size_t rollout_smem(const Consts& c, int block, bool single) {
+    return single && !extended(c) ? 0 : sizeof(float) * block * (2 * SMEM_PLANES + c.obs_dim + ROW_PAD);
+}
+
+int rollout_grid(const Consts& c, int block, bool single) {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, rollout_kernel(ext, single), block,
-                                                  sizeof(float) * 2 * SMEM_PLANES * block);
+    const void* fn = rollout_kernel(extended(c), single);
+    const size_t smem = rollout_smem(c, block, single);
+    allow_smem(fn, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
     return (occ > 0 ? occ : 1) * n_sm;
 }
 
@@ -1159,7 +1261,9 @@ cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, in
                            cudaStream_t st) {
     cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
     if (e != cudaSuccess) return e;
-    const size_t smem = sizeof(float) * 2 * SMEM_PLANES * block;
+    const size_t smem = rollout_smem(c, block, single);
+    e = allow_smem(rollout_kernel(extended(c), single), smem);
+    if (e != cudaSuccess) return e;
     const int g = grid > 0 ? grid : n_tiles;
     const int grid_n = g < n_tiles ? g : n_tiles;
     if (extended(c))
