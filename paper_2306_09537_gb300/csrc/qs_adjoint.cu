@@ -52,33 +52,44 @@ __device__ __forceinline__ float sigmoidf_(float z) {
 // (the acceleration itself is the substep's).
 __device__ __forceinline__ void wall_dacc(const Consts& c, const float x[3], float dacc[3]) {
     const float kcg = c.kc * c.g, b = c.beta;
-    dacc[0] = -kcg * (sigmoidf_(b * (-c.room_hx - x[0])) + sigmoidf_(b * (x[0] - c.room_hx)));
-    dacc[1] = -kcg * (sigmoidf_(b * (-c.room_hy - x[1])) + sigmoidf_(b * (x[1] - c.room_hy)));
-    dacc[2] = -kcg * (sigmoidf_(-b * x[2]) + sigmoidf_(b * (x[2] - c.room_h)));
+    const float z[6] = {b * (-c.room_hx - x[0]), b * (x[0] - c.room_hx), b * (-c.room_hy - x[1]),
+                        b * (x[1] - c.room_hy),  -b * x[2],              b * (x[2] - c.room_h)};
+    float sg[6];
+    // far from every face, the usual case: 1 + e rounds to 1 for e = exp(z) < 2^-24
+    if (fmaxf(fmaxf(fmaxf(z[0], z[1]), fmaxf(z[2], z[3])), fmaxf(z[4], z[5])) < -17.5f) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sg[k] = exp_approx(z[k]);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sg[k] = sigmoidf_(z[k]);
+    }
+    for (int k = 0; k < 3; ++k) dacc[k] = -kcg * (sg[2 * k] + sg[2 * k + 1]);
 }
 
 // lambda_x += sum_j J_ij (lam_a_i - lam_a_j)
 __device__ __forceinline__ void pair_vjp(const Consts& c, const float x[3], const float la[3], const float4* sp,
                                          const float* sla, int nt, int sbase, int lane, int N, float arm, float lx[3]) {
     const float kcg = c.kc * c.g, b = c.beta, far2 = pair_far_d2(arm, c.inv_beta);
-    for (int j = 0; j < N; ++j) {
-        if (j == lane) continue;
+    const auto dist2 = [&](int j) {
+        const float4 xj = sp[sbase + j];
+        const float r0 = x[0] - xj.x, r1 = x[1] - xj.y, r2 = x[2] - xj.z;
+        return r0 * r0 + r1 * r1 + r2 * r2;
+    };
+    near_pairs(lane, N, far2, dist2, [&](int j) {
         const int tj = sbase + j;
         const float4 xj = sp[tj];
         const float r0 = x[0] - xj.x, r1 = x[1] - xj.y, r2 = x[2] - xj.z;
-        const float d2 = r0 * r0 + r1 * r1 + r2 * r2;
-        if (d2 == 0.f || d2 > far2) continue;
-        const float d = sqrtf(d2), id = rcp_approx(d);
+        const float d = sqrtf(r0 * r0 + r1 * r1 + r2 * r2), id = rcp_approx(d);
         const float pen = 2.f * arm - d;
-        const float sp = softplus_b(pen, b, c.inv_beta), sg = sigmoidf_(b * pen);
-        const float psi = kcg * sp * id;
-        const float dpsi = kcg * (-sg * id - sp * id * id);  // d psi / d d
+        const float sp_ = softplus_b(pen, b, c.inv_beta), sg = sigmoidf_(b * pen);
+        const float psi = kcg * sp_ * id;
+        const float dpsi = kcg * (-sg * id - sp_ * id * id);  // d psi / d d
         const float q0 = la[0] - sla[tj], q1 = la[1] - sla[nt + tj], q2 = la[2] - sla[2 * nt + tj];
         const float rq = (r0 * q0 + r1 * q1 + r2 * q2) * dpsi * id;
         lx[0] += psi * q0 + rq * r0;
         lx[1] += psi * q1 + rq * r1;
         lx[2] += psi * q2 + rq * r2;
-    }
+    });
 }
 
 // Adjoint of R' = B(R Q(w1)) (Q the polar factor of I + dt [w1]x, B one
@@ -337,8 +348,14 @@ __device__ __forceinline__ bool group_sync_or(int id, int n, bool v) {
     if (id == 0) return __syncthreads_or(v) != 0;
     if (n == 32) return __any_sync(0xffffffffu, v);
     uint32_t r;
-    asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, %2, %3, p;\n selp.u32 %0, 1, 0, q;\n}"
-                 : "=r"(r) : "r"((uint32_t)v), "r"(id), "r"(n) : "memory");
+    // barrier numbers as immediates: with a number in a register the CTA is
+    // given all 16, and an SM's 64 then hold 4 CTAs
+    if (id == 1)
+        asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+                     : "=r"(r) : "r"((uint32_t)v), "r"(n) : "memory");
+    else
+        asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 2, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+                     : "=r"(r) : "r"((uint32_t)v), "r"(n) : "memory");
     return r != 0;
 }
 
@@ -397,9 +414,11 @@ struct DiffArgs {
     int T, C;
 };
 
-__device__ __forceinline__ void command4(const Consts& c, const float* act, size_t D, int t, int d, float fh[4], float u[4],
-                                         float msk[4]) {
-    const float4 a = __ldg(reinterpret_cast<const float4*>(act + (size_t)t * D * 4) + d);
+__device__ __forceinline__ float4 load_command(const float* act, size_t D, int t, int d) {
+    return __ldg(reinterpret_cast<const float4*>(act + (size_t)t * D * 4) + d);
+}
+
+__device__ __forceinline__ void command4(const Consts& c, const float4 a, float fh[4], float u[4], float msk[4]) {
     const float av[4] = {a.x, a.y, a.z, a.w};
     for (int r = 0; r < 4; ++r) {
         fh[r] = command(c, av[r]);
@@ -442,7 +461,11 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
         g[2] = dv.goal[2 * dv.E + e];
     }
     float L = 0.f;
+    // the commands of step t + 1 are loaded while step t integrates
+    float4 cmd = act ? load_command(a.act, D, 0, d) : make_float4(0.f, 0.f, 0.f, 0.f);
     for (int t = 0; t < a.T; ++t) {
+        const float4 at = cmd;
+        if (act && t + 1 < a.T) cmd = load_command(a.act, D, t + 1, d);
         __syncthreads();  // step t's motor normals ready (group 1)
         if (act && t % a.C == 0) {
             float4 q[NPLANE];
@@ -451,7 +474,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
             for (int pl = 0; pl < NPLANE; ++pl) ck[(size_t)pl * D + d] = q[pl];
         }
         float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f}, msk[4];
-        if (act) command4(c, a.act, D, t, d, fh, u, msk);
+        if (act) command4(c, at, fh, u, msk);
         for (int sub = 0; sub < c.substeps; ++sub) {
             float n[4];
             if (ahead)
@@ -478,7 +501,15 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
 // synchronises its staged positions with its own barrier. The reverse takes
 // each substep's updated motor noise (and each step's end position) from the
 // next saved input instead of drawing it again.
-__global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
+//
+// Bound by the chain of the reverse substeps with one warp of each group a
+// scheduler (1024 x 8 drones, 128 steps: forward 532 -> 382 us and reverse 646
+// -> 466 us with the near pairs and the room's faces tested ahead of their rare
+// branches and commands loaded a step ahead).
+// DENSE: 64-thread CTAs held to 168 registers (a few spills), six an SM
+// instead of four, for batches of several waves (dense_backward()).
+template <bool DENSE>
+__global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_diff_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                             const int* __restrict__ perm, const DiffArgs a) {
     extern __shared__ float4 sm4[];
     float* sm = reinterpret_cast<float*>(sm4);
@@ -523,9 +554,12 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, cons
                 for (int pl = 0; pl < NPLANE; ++pl) q[pl] = ck[(size_t)pl * D + d];
                 unpack(s, q);
             }
+            float4 cmd = act ? load_command(a.act, D, tb, d) : make_float4(0.f, 0.f, 0.f, 0.f);
             for (int t = tb; t < te; ++t) {
+                const float4 at = cmd;
+                if (act && t + 1 < te) cmd = load_command(a.act, D, t + 1, d);
                 float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f}, msk[4];
-                if (act) command4(c, a.act, D, t, d, fh, u, msk);
+                if (act) command4(c, at, fh, u, msk);
                 for (int sub = 0; sub < S; ++sub) {
                     if (act) save_sub(scr, D, (t - tb) * S + sub, d, s);
                     smooth_substep(c, s, p, u, tick0 + t, d, sub, act, sp, sbase, lane, N, lt, bid, nb);
@@ -541,12 +575,15 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_bwd(const Consts c, cons
             const int seg = nseg - it, tb = seg * a.C, te = min(a.T, tb + a.C);
             const float* scr = a.scratch + (size_t)((it - 1) & 1) * sbuf;
             const float* f = fin + ((it - 1) & 1) * 7 * nb;
+            float4 cmd = act ? load_command(a.act, D, te - 1, d) : make_float4(0.f, 0.f, 0.f, 0.f);
             for (int t = te - 1; t >= tb; --t) {
+                const float4 at = cmd;
+                if (act && t > tb) cmd = load_command(a.act, D, t - 1, d);
                 float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f}, msk[4] = {0.f, 0.f, 0.f, 0.f};
                 // the state after step t: the next step's first input, or the segment's end
                 float xpost[3] = {0.f, 0.f, 0.f}, eps_end[4] = {0.f, 0.f, 0.f, 0.f};
                 if (act) {
-                    command4(c, a.act, D, t, d, fh, u, msk);
+                    command4(c, at, fh, u, msk);
                     if (t + 1 < te) {
                         load_x(scr, D, (t + 1 - tb) * S, d, xpost);
                         load_eps(scr, D, (t + 1 - tb) * S, d, eps_end);
@@ -682,9 +719,6 @@ __device__ __forceinline__ void discrete_substep_vjp(const Drone& s, const Prm& 
         pass[k] = fabsf(hi) > c.omega_max ? 0.f : 1.f;
         w1[k] = fabsf(hi) > c.omega_max ? copysignf(c.omega_max, hi) : hi;
     }
-    float R1[9];
-    for (int k = 0; k < 9; ++k) R1[k] = s.R[k];
-    rotate_polar(R1, w1, dt);
     const bool hit = (c.flags & QS_F_FLOOR) && x1[2] <= 0.0f && v1[2] < 0.0f;
     // event-time floor: crossing time and the velocity that led there
     float tf = dt, vz_hit = 0.f;
@@ -760,6 +794,9 @@ __device__ __forceinline__ void discrete_substep_vjp(const Drone& s, const Prm& 
         lw[0] = lw[1] = lw[2] = 0.0f;
         const float lcs = lR[0] + lR[4], lsn = lR[3] - lR[1];
         for (int k = 0; k < 9; ++k) lR[k] = 0.0f;
+        float R1[9];  // the attitude the hit reset
+        for (int k = 0; k < 9; ++k) R1[k] = s.R[k];
+        rotate_polar(R1, w1, dt);
         const float h2 = R1[0] * R1[0] + R1[3] * R1[3];
         if (h2 >= 1e-12f) {  // cs = R0 / h, sn = R3 / h
             const float ih = rsqrtf(h2), ih3 = ih * ih * ih;
@@ -1179,7 +1216,11 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
     }
     const float zero3[3] = {0.f, 0.f, 0.f};
     float L = 0.f;
+    // the commands of step t + 1 are loaded while step t integrates
+    float4 cmd = act ? load_command(a.act, D, 0, d) : make_float4(0.f, 0.f, 0.f, 0.f);
     for (int t = 0; t < a.T; ++t) {
+        const float4 at = cmd;
+        if (act && t + 1 < a.T) cmd = load_command(a.act, D, t + 1, d);
         __syncthreads();  // step t's motor normals ready (group 1)
         if (act && t % a.C == 0) {
             float4 q[NPLANE];
@@ -1189,7 +1230,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
         }
         float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f}, msk[4];
         if (act) {
-            command4(c, a.act, D, t, d, fh, u, msk);
+            command4(c, at, fh, u, msk);
             for (int sub = 0; sub < c.substeps; ++sub) {
                 float n[4];
                 if (ahead)
@@ -1214,8 +1255,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
 // like k_diff_bwd: group 0 recomputes segment s - 1 (every substep input and
 // each step's pre-collision state) into one scratch buffer while group 1
 // reverses segment s from the other.
-template <bool ET>
-__global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
+template <bool ET, bool DENSE>
+__global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_diffd_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                              const int* __restrict__ perm, const DiffArgs a) {
     extern __shared__ float4 sm4[];
     float* sm = reinterpret_cast<float*>(sm4);
@@ -1273,10 +1314,13 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
                 for (int pl = 0; pl < NPLANE; ++pl) q[pl] = ck[(size_t)pl * D + d];
                 unpack(s, q);
             }
+            float4 cmd = act ? load_command(a.act, D, tb, d) : make_float4(0.f, 0.f, 0.f, 0.f);
             for (int t = tb; t < te; ++t) {
+                const float4 at = cmd;
+                if (act && t + 1 < te) cmd = load_command(a.act, D, t + 1, d);
                 float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f}, msk[4];
                 if (act) {
-                    command4(c, a.act, D, t, d, fh, u, msk);
+                    command4(c, at, fh, u, msk);
                     for (int sub = 0; sub < S; ++sub) {
                         save_sub(scr, D, (t - tb) * S1 + sub, d, s);
                         substep<ET, 0>(s, p, c, u, tick0 + t, d, sub, zero3);
@@ -1295,13 +1339,16 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
             const int seg = nseg - it, tb = seg * a.C, te = min(a.T, tb + a.C);
             const float* scr = a.scratch + (size_t)((it - 1) & 1) * sbuf;
             const uint32_t* fl = rflag + ((it - 1) & 1) * RFLAG_WORDS;
+            float4 cmd = act ? load_command(a.act, D, te - 1, d) : make_float4(0.f, 0.f, 0.f, 0.f);
             for (int t = te - 1; t >= tb; --t) {
+                const float4 at = cmd;
+                if (act && t > tb) cmd = load_command(a.act, D, t - 1, d);
                 const int q = t - tb;  // the same in every thread of the group
                 const bool any = q >= RFLAG_BITS || ((fl[q >> 5] >> (q & 31)) & 1u);
                 float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f}, msk[4] = {0.f, 0.f, 0.f, 0.f};
                 Drone sc;
                 if (act) {
-                    command4(c, a.act, D, t, d, fh, u, msk);
+                    command4(c, at, fh, u, msk);
                     load_sub(scr, D, (t - tb) * S1 + S, d, sc);
                     // loss of step t: |x(t) - g|^2 + 1e-3 |f^|^2 (the collision pass leaves x
                     // unchanged; the event-time pass moves it and adds the term itself)
@@ -1357,6 +1404,21 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_bwd(const Consts c, con
     }
 }
 
+// Whether the backward pass of n_tiles CTAs takes the instance with six CTAs an
+// SM: its wave takes 1.25 times as long as one of four (64-thread CTAs), so it
+// pays where it saves enough waves. Measured, forward and backward, discrete
+// contacts, swarms of 8: 2400 envs (600 CTAs, one wave either way) 500 us
+// without and 530 with it; 8192 envs, 64 steps, 1612 and 1535; 32768 envs, 16
+// steps, 1480 and 1330. (Seven an SM, 128 registers: 635, 1571, 1418.)
+bool dense_backward(int n_tiles, int block) {
+    if (block != 32) return false;
+    int dev = 0, n_sm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    const long w4 = (n_tiles + 4L * n_sm - 1) / (4L * n_sm), w6 = (n_tiles + 6L * n_sm - 1) / (6L * n_sm);
+    return 5 * w6 < 4 * w4;
+}
+
 cudaError_t launch_diff(int backward, const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int block,
                         const int* perm, const float* x0, const float* act, float* loss, const float* dloss,
                         float* grad_act, float* grad_x0, void* workspace, int T, int C, cudaStream_t st) {
@@ -1377,15 +1439,16 @@ cudaError_t launch_diff(int backward, const Consts& c, const Dev& dv, const Tile
     const size_t smem = sizeof(float) * (7 + 2 * FWD_SUB * 4) * block,
                  smem2 = sizeof(float) * BWD_PLANES * block + sizeof(uint32_t) * 2 * RFLAG_WORDS;
     if (2 * block > ADJ_BLOCK_MAX) return cudaErrorInvalidValue;
-    if (c.flags & QS_F_SMOOTH) {
-        if (backward) k_diff_bwd<<<n_tiles, 2 * block, smem2, st>>>(c, dv, tiles, perm, a);
-        else k_diff_fwd<<<n_tiles, 2 * block, smem, st>>>(c, dv, tiles, perm, a);
-    } else if (c.flags & QS_F_EVENT_TIME) {
-        if (backward) k_diffd_bwd<true><<<n_tiles, 2 * block, smem2, st>>>(c, dv, tiles, perm, a);
-        else k_diffd_fwd<true><<<n_tiles, 2 * block, smem, st>>>(c, dv, tiles, perm, a);
+    const bool smooth = (c.flags & QS_F_SMOOTH) != 0, et = !smooth && (c.flags & QS_F_EVENT_TIME) != 0;
+    if (backward) {
+        const bool dense = dense_backward(n_tiles, block);
+        const auto k = smooth ? (dense ? k_diff_bwd<true> : k_diff_bwd<false>)
+                       : et   ? (dense ? k_diffd_bwd<true, true> : k_diffd_bwd<true, false>)
+                              : (dense ? k_diffd_bwd<false, true> : k_diffd_bwd<false, false>);
+        k<<<n_tiles, 2 * block, smem2, st>>>(c, dv, tiles, perm, a);
     } else {
-        if (backward) k_diffd_bwd<false><<<n_tiles, 2 * block, smem2, st>>>(c, dv, tiles, perm, a);
-        else k_diffd_fwd<false><<<n_tiles, 2 * block, smem, st>>>(c, dv, tiles, perm, a);
+        const auto k = smooth ? k_diff_fwd : et ? k_diffd_fwd<true> : k_diffd_fwd<false>;
+        k<<<n_tiles, 2 * block, smem, st>>>(c, dv, tiles, perm, a);
     }
     return cudaGetLastError();
 }

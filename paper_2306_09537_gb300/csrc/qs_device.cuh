@@ -457,6 +457,31 @@ __device__ __forceinline__ float pair_far_d2(float arm, float inv_beta) {
     return r * r;
 }
 
+// Calls body(j), in increasing j, for every partner j of the thread's drone with
+// d2(j) between 0 and far2 (pair_far_d2). Most swarms have no such pair in most
+// substeps, so the distances of 32 partners are tested first, four at a time
+// and without a branch between them, and only the near ones are visited.
+template <class D2, class Body>
+__device__ __forceinline__ void near_pairs(int lane, int N, float far2, const D2& d2, const Body& body) {
+    for (int j0 = 0; j0 < N; j0 += 32) {
+        uint32_t near = 0;
+        const int n = min(N - j0, 32);
+        for (int i = 0; i < n; i += 4) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int j = j0 + i + q;
+                const float v = d2(min(j, N - 1));
+                if (!(v == 0.f || v > far2) && j != lane && j < N) near |= 1u << (i + q);
+            }
+        }
+        while (near) {
+            const int i = __ffs(near) - 1;
+            near &= near - 1;
+            body(j0 + i);
+        }
+    }
+}
+
 // Smooth pair acceleration of the thread's drone from the slot's positions in
 // shared memory (sp: one float4 a drone); j == lane and coincident drones
 // contribute 0.
@@ -464,18 +489,47 @@ __device__ __forceinline__ void pair_acc(const Consts& c, const float x[3], cons
                                          float arm, float out[3]) {
     out[0] = out[1] = out[2] = 0.f;
     const float kcg = __fmul_rn(c.kc, c.g), far2 = pair_far_d2(arm, c.inv_beta);
-    for (int j = 0; j < N; ++j) {
-        if (j == lane) continue;
+    const auto dist2 = [&](int j) {
         const float4 q = sp[sbase + j];
         const float r0 = x[0] - q.x, r1 = x[1] - q.y, r2 = x[2] - q.z;
-        const float d2 = __fmaf_rn(r2, r2, __fmaf_rn(r1, r1, __fmul_rn(r0, r0)));
-        if (d2 == 0.f || d2 > far2) continue;
-        const float d = sqrtf(d2);
+        return __fmaf_rn(r2, r2, __fmaf_rn(r1, r1, __fmul_rn(r0, r0)));
+    };
+    near_pairs(lane, N, far2, dist2, [&](int j) {
+        const float4 q = sp[sbase + j];
+        const float r0 = x[0] - q.x, r1 = x[1] - q.y, r2 = x[2] - q.z;
+        const float d = sqrtf(__fmaf_rn(r2, r2, __fmaf_rn(r1, r1, __fmul_rn(r0, r0))));
         const float psi = __fmul_rn(__fmul_rn(kcg, softplus_b(__fsub_rn(2.f * arm, d), c.beta, c.inv_beta)), __frcp_rn(d));
         out[0] = fmaf(psi, r0, out[0]);
         out[1] = fmaf(psi, r1, out[1]);
         out[2] = fmaf(psi, r2, out[2]);
+    });
+}
+
+// Softplus penalties of the six faces of the room, opposite faces subtracted:
+// (low - high) per axis. A drone more than 16 / beta from every face, the usual
+// case, takes all six in one straight run (the first branch of softplus_b).
+__device__ __forceinline__ void room_softplus(const Consts& c, const float x[3], float out[3]) {
+    const float b = c.beta, ib = c.inv_beta;
+    const float u[6] = {__fsub_rn(-c.room_hx, x[0]), __fsub_rn(x[0], c.room_hx), __fsub_rn(-c.room_hy, x[1]),
+                        __fsub_rn(x[1], c.room_hy),  -x[2],                      __fsub_rn(x[2], c.room_h)};
+    const float top = __fmul_rn(b, fmaxf(fmaxf(fmaxf(u[0], u[1]), fmaxf(u[2], u[3])), fmaxf(u[4], u[5])));
+    float sp[6];
+    if (top < -16.0f) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) sp[k] = __fmul_rn(exp_approx(__fmul_rn(b, u[k])), ib);
+    } else {
+#pragma unroll 1
+        for (int k = 0; k < 6; k += 2) {
+            const float lo = softplus_b(k == 0 ? u[0] : k == 2 ? u[2] : u[4], b, ib);
+            const float hi = softplus_b(k == 0 ? u[1] : k == 2 ? u[3] : u[5], b, ib);
+            if (k == 0) { sp[0] = lo; sp[1] = hi; }
+            if (k == 2) { sp[2] = lo; sp[3] = hi; }
+            if (k == 4) { sp[4] = lo; sp[5] = hi; }
+        }
     }
+    out[0] = __fsub_rn(sp[0], sp[1]);
+    out[1] = __fsub_rn(sp[2], sp[3]);
+    out[2] = __fsub_rn(sp[4], sp[5]);
 }
 
 // R <- polar(R + dt R [w]x) for a rotation R. In closed form the polar factor
@@ -576,15 +630,11 @@ __device__ __forceinline__ uint32_t substep(Drone& s, const Prm& p, const Consts
     bool on_floor = false, moving = false;
     if (smooth) {  // explicit roundings (see softplus_b)
         const float kcg = __fmul_rn(c.kc, g);
-        const float b = c.beta, ib = c.inv_beta;
-        const float pz = __fsub_rn(softplus_b(-s.x[2], b, ib), softplus_b(__fsub_rn(s.x[2], c.room_h), b, ib));
-        const float px = __fsub_rn(softplus_b(__fsub_rn(-c.room_hx, s.x[0]), b, ib),
-                                   softplus_b(__fsub_rn(s.x[0], c.room_hx), b, ib));
-        const float py = __fsub_rn(softplus_b(__fsub_rn(-c.room_hy, s.x[1]), b, ib),
-                                   softplus_b(__fsub_rn(s.x[1], c.room_hy), b, ib));
-        a2 = __fadd_rn(__fmaf_rn(kcg, pz, a2), pacc[2]);
-        a0 = __fadd_rn(__fmaf_rn(kcg, px, a0), pacc[0]);
-        a1 = __fadd_rn(__fmaf_rn(kcg, py, a1), pacc[1]);
+        float pw[3];
+        room_softplus(c, s.x, pw);
+        a0 = __fadd_rn(__fmaf_rn(kcg, pw[0], a0), pacc[0]);
+        a1 = __fadd_rn(__fmaf_rn(kcg, pw[1], a1), pacc[1]);
+        a2 = __fadd_rn(__fmaf_rn(kcg, pw[2], a2), pacc[2]);
     } else if ((c.flags & QS_F_FLOOR) && s.x[2] <= 0.0f) {
         const float mg = __fmul_rn(p.m, g);
         if (F2 < mg) {
