@@ -302,7 +302,8 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
  * kernel (32..256, a multiple of 32, at least the widest swarm class), or
  * QS_BLOCK_WARP_SPECIALISED (every class at most 64 wide; the default when
  * every class is at most 32 wide, all of the handle's such CTAs are
- * resident at once and neither scenarios nor downwash are on): per 32 drones
+ * resident at once, up to five an SM for classes of 17..32, and with
+ * scenarios or downwash when there is one class): per 32 drones
  * (64 when a class is wider than 32) one CTA whose dynamics warps integrate
  * while as many noise warps draw the noise and store the observation rows,
  * every step; `fuse` control steps per

@@ -522,17 +522,18 @@ qs_status qs_create(const qs_config* cfg, void* cuda_stream, qs_env** out) {
         }
     }
     // default rollout shape: warp-specialised while every class is at most 32
-    // wide, its CTAs (one per 32 drone lanes) fit one wave on the device
-    // (latency-bound; a second wave would run the whole horizon again) and
-    // neither scenarios nor downwash lengthen the dynamics warp's step (then
-    // its noise warp would idle at the barriers); else the persistent kernel,
-    // whose work counter also balances uneven swarm sizes. Measured on GB300
-    // (warp-specialised vs persistent, us per step): plain 8192 x 1 2.66 vs
-    // 3.47, 28,672 x 1 3.75 vs 3.90, 30,720 x 1 (past the 29,184 lanes of
-    // one wave) 5.89 vs 3.90; swarm 2048 x 8 4.81 vs 6.67, 4096 x 8 9.46 vs
-    // 7.81; with every scenario type 1.9e9 vs 2.0e9 quadrotor-steps/s;
-    // uneven sizes up to 64 (two-warp pairs per CTA) 1.86e9 vs 1.80e9, close
-    // enough to leave to the autotuner.
+    // wide and its CTAs (one per 32 drone lanes) fit one wave on the device
+    // (latency-bound; a second wave would run the whole horizon again), for
+    // classes of 17..32 up to five CTAs an SM (their pair pass fills the issue
+    // slots the noise warps would use); else the persistent kernel, whose work
+    // counter also balances uneven swarm sizes. Scenarios and downwash take it
+    // when there is one class. Measured on GB300 (warp-specialised vs
+    // persistent, us per step): plain 8192 x 1 1.92 vs 2.21, 28,672 x 1 2.63 vs
+    // 2.69, 30,720 x 1 (past the 29,184 lanes of one wave) 4.00 vs 2.69; swarm
+    // 2048 x 8 3.44 vs 4.48, 3600 x 8 4.31 vs 4.98, 4096 x 8 6.95 vs 5.02; 600 x
+    // 32 5.27 vs 5.73, 900 x 32 6.69 vs 6.56; under every scenario with downwash
+    // 1999 x 7 4.42 vs 5.67, 3000 x 8 4.93 vs 6.17, 600 x 32 7.37 vs 7.89, 900 x
+    // 32 9.81 vs 8.98.
     {
         int maxW = 1;
         long ws_ctas = 0;
@@ -542,7 +543,8 @@ qs_status qs_create(const qs_config* cfg, void* cuda_stream, qs_env** out) {
             ws_ctas += (h->class_slots[ci] + per - 1) / per;
         }
         const bool ext = (h->c.scn_mask & ~1u) != 0 || (h->c.flags & QS_F_DOWNWASH) != 0;
-        if (maxW <= 32 && !ext && ws_ctas <= rollout_ws_resident_ctas(h->c, 1))
+        if (maxW <= 32 && (!ext || h->plan.size() == 1) && ws_ctas <= rollout_ws_resident_ctas(h->c, 1) &&
+            (maxW <= 16 || ws_ctas <= 5L * n_sm))
             h->rollout_block = QS_BLOCK_WARP_SPECIALISED;
     }
 

@@ -34,7 +34,7 @@ constexpr int SMEM_PLANES = 8;
 // the padding of its block (RowMap)
 constexpr int ROW_PAD = 6;
 // and the most the kernels ask for
-constexpr int STEP_SMEM_MAX = (int)sizeof(float) * MAX_BLOCK * (2 * SMEM_PLANES + 18 + 6 * QS_MAX_K + ROW_PAD);
+constexpr int STEP_SMEM_MAX = (int)sizeof(float) * MAX_BLOCK * (2 * SMEM_PLANES + GOAL_STRIDE + 18 + 6 * QS_MAX_K + ROW_PAD);
 
 // The step kernels come in two instances: EXT = true carries the training
 // scenarios (per-drone goals), the downwash term and the smooth contacts,
@@ -360,15 +360,9 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
     // ---- the drone's goal at the end of the step (Sec. III-D scenarios)
     float gl[3] = {er.g0, er.g1, er.g2};
     if (scn && act) {
-        if (goal_cached(gc, tau)) {
-            gl[0] = gc.g[0];
-            gl[1] = gc.g[1];
-            gl[2] = gc.g[2];
-        } else {
-            const int slot = swp ? swap_rank(skey, sbase, N, lane, myk) : lane;
-            scenario_goal(c, dv, er.sel, e, lane, N, tau, slot, gl, gl);
-            goal_cache_set(gc, dv, er.sel, e, tau, gl);
-        }
+        if (!goal_cached(gc, tau))
+            goal_fill(gc, c, dv, er.sel, e, lane, N, tau, swp ? swap_rank(skey, sbase, N, lane, myk) : lane, gl);
+        goal_at(gc, c, tau, gl);
     }
 
     // ---- S12 observation
@@ -460,7 +454,8 @@ __global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Cons
     }
     const float4 a = (m.act && !observe_only) ? __ldg(reinterpret_cast<const float4*>(io.act) + m.d)
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
-    GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
+    float gv[GOAL_VALUES];
+    GoalCache gc{gv, GOAL_FIXED, 0, -1};
     step_body<EXT, false>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
               io.rew, io.done, observe_only, gc, RowMap(), nullptr, false);
     if (!m.act || observe_only) return;
@@ -489,9 +484,10 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
     // the commands of step t + 1 are loaded while step t computes, so their
     // HBM latency leaves each step's dependent chain
     float4 a_next = m.act ? __ldg(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
-    GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
+    float* goals = reinterpret_cast<float*>(sm + 2 * SMEM_PLANES / 4 * blockDim.x);  // the general instance's goal values
+    GoalCache gc{goals + GOAL_STRIDE * threadIdx.x, GOAL_FIXED, 0, -1};
     const RowMap rm = W1 ? RowMap() : map_rows(m.act, m.d, W, c.obs_dim);
-    float* rows = reinterpret_cast<float*>(sm + 2 * SMEM_PLANES / 4 * blockDim.x) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
+    float* rows = goals + (EXT ? GOAL_STRIDE * blockDim.x : 0) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
     for (int t = t0; t < t0 + nsteps; ++t) {
         const float4 a = a_next;
         if (m.act && t + 1 < t0 + nsteps) a_next = __ldg(act4 + (size_t)(t + 1) * D);
@@ -555,13 +551,14 @@ struct WsShared {
     // the published end of a step, [buffer] by step parity:
     float st[2][18][32 * P];          // x v R w of each drone lane after the step (post-collision)
     float g[2][3][32 * P];            // goal of each lane's drone
-    int nb[2][QS_MAX_K][32 * P];      // CTA drone lane of each neighbour
+    NbrList nb[2][32 * P];            // CTA drone lanes of the neighbours
     int keff[2][32 * P];
     float rin[2][9][32 * P];          // reward inputs: command f^ (4), previous command (4), proximity radius
     uint32_t ev[2][32 * P];           // event bits
     float4 sp[32 * P];                // pair-pass staging: positions
     float sv[3][32 * P];              //                    velocities
     uint32_t key[32 * P];             // swap keys
+    float gv[32 * P][GOAL_STRIDE];    // goal values of each lane's drone (GoalCache)
     float rows[32 * P * WS_OBS_MAX];
 };
 
@@ -644,10 +641,11 @@ __device__ __forceinline__ void ws_store_obs(const Consts& c, const Dev& dv, con
         row[16] = st[16][L] + ew[1];
         row[17] = st[17][L] + ew[2];
         const int ke = sh.keff[b][L];
+        const NbrList nb = sh.nb[b][L];
         for (int k = 0; k < K; ++k) {
             float* on = row + 18 + 6 * k;
             if (k < ke) {
-                const int j = sh.nb[b][k][L];
+                const int j = nbr_at(nb, k);
                 for (int q = 0; q < 6; ++q) on[q] = st[q][j] - st[q][L];
             } else {
                 for (int q = 0; q < 6; ++q) on[q] = 0.f;
@@ -677,6 +675,29 @@ __device__ __forceinline__ void ws_store_obs(const Consts& c, const Dev& dv, con
         float2* dst2 = reinterpret_cast<float2*>(obs + (size_t)m.d * od);
         for (int i = 0; i < od / 2; ++i) dst2[i] = src2[i];
     }
+}
+
+// The goal of the lane's drone at control step tau under the scenario record in
+// buffer sel (Sec. III-D scenarios); gl holds the env's single goal on entry.
+// Every thread of the side (side_sync id) calls it.
+template <int P>
+__device__ __forceinline__ void ws_goal(const Consts& c, const Dev& dv, WsShared<P>& sh, const WsMap& m, int sel, int tau,
+                                        GoalCache& gc, float gl[3], int id) {
+    const bool hit = goal_cached(gc, tau);  // the same for every lane of an env
+    bool swp = false;
+    uint32_t myk = 0;
+    if (m.W > 1) {
+        if (m.act && !hit && swap_active(dv, sel, m.e, tau)) {
+            swp = true;
+            myk = swap_key(c, scn_seed(dv, sel, m.e), m.lane);
+            sh.key[m.L] = myk;
+        }
+        side_sync<P>(id);
+    }
+    if (!m.act) return;
+    if (!hit)
+        goal_fill(gc, c, dv, sel, m.e, m.lane, m.N, tau, swp ? swap_rank(sh.key, m.sbase, m.N, m.lane, myk) : m.lane, gl);
+    goal_at(gc, c, tau, gl);
 }
 
 // Dynamics side: one control step of the lane's drone with command a and the
@@ -763,31 +784,10 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         if (responded) apply_response(c, s, er.tick, d, dvs);
         if (dw && dw_hit) apply_downwash(c, s, er.tick, d, dw_az);
     }
-    // the drone's goal at the end of the step (Sec. III-D scenarios)
+    // the drone's goal at the end of the step; in the rollout the noise side
+    // evaluates it
     float gl[3] = {er.g0, er.g1, er.g2};
-    if (EXT && (c.scn_mask & ~1u)) {
-        const int tau = er.ep + 1;
-        const bool hit = goal_cached(gc, tau);  // the same for every lane of an env
-        bool swp = false;
-        uint32_t myk = 0;
-        if (W > 1) {
-            if (act && !hit && swap_active(dv, er.sel, e, tau)) {
-                swp = true;
-                myk = swap_key(c, scn_seed(dv, er.sel, e), lane);
-                sh.key[L] = myk;
-            }
-            side_sync<P>(1);
-        }
-        if (act && hit) {
-            gl[0] = gc.g[0];
-            gl[1] = gc.g[1];
-            gl[2] = gc.g[2];
-        } else if (act) {
-            const int slot = swp ? swap_rank(sh.key, sbase, N, lane, myk) : lane;
-            scenario_goal(c, dv, er.sel, e, lane, N, tau, slot, gl, gl);
-            goal_cache_set(gc, dv, er.sel, e, tau, gl);
-        }
-    }
+    if (EXT && !DEFER && (c.scn_mask & ~1u)) ws_goal<P>(c, dv, sh, m, er.sel, er.ep + 1, gc, gl, 1);
     if (act) {  // publish the observed state (post-collision) for the noise side
         const float v18[18] = {s.x[0], s.x[1], s.x[2], s.v[0], s.v[1], s.v[2], s.R[0], s.R[1], s.R[2],
                                s.R[3], s.R[4], s.R[5], s.R[6], s.R[7], s.R[8], s.w[0], s.w[1], s.w[2]};
@@ -797,9 +797,7 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         sh.g[b][1][L] = gl[1];
         sh.g[b][2][L] = gl[2];
         sh.keff[b][L] = W > 1 ? keff : 0;
-#pragma unroll
-        for (int k = 0; k < QS_MAX_K; ++k)
-            if (k < keff) sh.nb[b][k][L] = sbase + nbr_at(nbrs, k);
+        sh.nb[b][L] = nbrs + (NbrList)sbase * 0x0101010101010101ull;  // (fields past keff are not read)
         if (DEFER) {  // the noise side computes the reward from these
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -823,7 +821,7 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
             return make_float3(q.x, q.y, q.z);
         });
     end_step<EXT>(c, dv, s, er, fh, lane, e, d, done);
-    if (EXT && er.ep == 0) gc.until = -1;  // an auto-reset drew a new record
+    if (EXT && !DEFER && er.ep == 0) gc.until = -1;  // an auto-reset drew a new record
     ev_out = ev;
 }
 
@@ -847,8 +845,9 @@ __device__ __forceinline__ void ws_reward(const Consts& c, WsShared<P>& sh, cons
         s.fp[r] = sh.rin[b][4 + r][L];
     }
     const float g[3] = {sh.g[b][0][L], sh.g[b][1][L], sh.g[b][2][L]};
+    const NbrList nb = sh.nb[b][L];
     rew[m.d] = compute_reward(c, s, sh.rin[b][8][L], g, fh, sh.ev[b][L], sh.keff[b][L], [&](int k) {
-        const int j = sh.nb[b][k][L];
+        const int j = nbr_at(nb, k);
         return make_float3(sh.st[b][0][j], sh.st[b][1][j], sh.st[b][2][j]);
     });
 }
@@ -880,7 +879,7 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
         load_env<EXT>(er, c, dv, m.e);
         a = __ldg(reinterpret_cast<const float4*>(io.act) + m.d);
     }
-    GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
+    GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
     ws_dynamics_step<EXT, 1, false>(c, dv, sh, m, s, er, ev, a, 0, io.rew, io.done, gc);
     if (!m.act) return;
     dv.ev[m.d] = ev;
@@ -914,6 +913,30 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
         const uint32_t tick0 = m.act ? dv.tick[m.e] : 0u;  // the dynamics side writes it after the last step
         ws_motor_normals<P>(c, sh, m, tick0, 0);
         float px[3] = {0.f, 0.f, 0.f}, pv[3] = {0.f, 0.f, 0.f}, pw[3] = {0.f, 0.f, 0.f};  // step t-1's sensor noise
+        // scenario goals: the episode step and record buffer of the step being
+        // finished, advanced as the dynamics side advances them. A record is
+        // drawn after B2 of the step that ends its predecessor's episode, into
+        // the other buffer, and first read after the next B2.
+        const bool scn = EXT && (c.scn_mask & ~1u) != 0;
+        int ep = scn && m.act ? dv.ep[m.e] : 0, sel = scn && m.act ? dv.scn_sel[m.e] : 0;
+        GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
+        // finishes the step published in buffer b (time t0 + t): goals, rows, rewards
+        const auto finish = [&](int t) {
+            const int b = t & 1;
+            if (scn) {
+                float gl[3] = {sh.g[b][0][m.L], sh.g[b][1][m.L], sh.g[b][2][m.L]};
+                ws_goal<P>(c, dv, sh, m, sel, ep + 1, gc, gl, 2);
+                for (int k = 0; k < 3; ++k) sh.g[b][k][m.L] = gl[k];
+                ep = ep + 1;
+                if (ep >= c.episode_steps && (c.flags & QS_F_AUTO_RESET)) {
+                    ep = 0;
+                    sel ^= 1;
+                    gc.until = -1;
+                }
+            }
+            if (io.obs) ws_store_obs<P>(c, dv, tile, perm, sh, m, b, io.obs + (size_t)(t0 + t) * D * c.obs_dim, px, pv, pw);
+            if (io.rew) ws_reward<P>(c, sh, m, b, io.rew + (size_t)(t0 + t) * D);
+        };
         for (int t = 0; t < nsteps; ++t) {
             // buffer t & 1 holds step t's normals, drawn before B2 of step t - 1:
             // B1 is needed before the first step only; swarm slots (whose
@@ -925,12 +948,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
             if (m.act && io.obs && (c.flags & QS_F_OBS_NOISE)) obs_noise(c, tick, m.d, 0u, ex, evv, ew);
             // the other buffer was last read by the dynamics side before B2 of step t - 1
             if (t + 1 < nsteps) ws_motor_normals<P>(c, sh, m, tick + 1, (t + 1) & 1);
-            if (t > 0) {
-                const int pb = (t - 1) & 1;
-                if (io.obs) ws_store_obs<P>(c, dv, tile, perm, sh, m, pb, io.obs + (size_t)(t0 + t - 1) * D * c.obs_dim,
-                                            px, pv, pw);
-                if (io.rew) ws_reward<P>(c, sh, m, pb, io.rew + (size_t)(t0 + t - 1) * D);
-            }
+            if (t > 0) finish(t - 1);
             for (int k = 0; k < 3; ++k) {
                 px[k] = ex[k];
                 pv[k] = evv[k];
@@ -938,12 +956,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
             }
             __syncthreads();  // B2 of step t
         }
-        if (nsteps > 0) {  // the last step, after its B2
-            const int pb = (nsteps - 1) & 1;
-            if (io.obs)
-                ws_store_obs<P>(c, dv, tile, perm, sh, m, pb, io.obs + (size_t)(t0 + nsteps - 1) * D * c.obs_dim, px, pv, pw);
-            if (io.rew) ws_reward<P>(c, sh, m, pb, io.rew + (size_t)(t0 + nsteps - 1) * D);
-        }
+        if (nsteps > 0) finish(nsteps - 1);  // after the last B2
         return;
     }
     // ---------------- dynamics side
@@ -956,7 +969,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
     }
     const float4* act4 = reinterpret_cast<const float4*>(io.act) + m.d;
     float4 a_next = m.act ? __ldg(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
-    GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
+    GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
     for (int t = 0; t < nsteps; ++t) {
         const float4 a = a_next;
         if (m.act && t + 1 < nsteps) a_next = __ldg(act4 + (size_t)(t0 + t + 1) * D);
@@ -1083,7 +1096,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_serve(const Consts
     Drone s;
     EnvRegs er;
     uint32_t ev = 0;
-    GoalCache gc{{0.f, 0.f, 0.f}, 0, -1};
+    GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
     if (!noise && m.act) {
         load_drone(s, dv.st, dv.D, m.d);
         load_env<EXT>(er, c, dv, m.e);
@@ -1222,7 +1235,8 @@ cudaError_t allow_smem(const void* fn, size_t smem) {
 // Its dynamic shared memory: two sets of staging planes and the CTA's
 // observation rows (none for single drones).
 size_t rollout_smem(const Consts& c, int block, bool single) {
-    return single && !extended(c) ? 0 : sizeof(float) * block * (2 * SMEM_PLANES + c.obs_dim + ROW_PAD);
+    const bool ext = extended(c);
+    return single && !ext ? 0 : sizeof(float) * block * (2 * SMEM_PLANES + (ext ? GOAL_STRIDE : 0) + c.obs_dim + ROW_PAD);
 }
 
 int rollout_grid(const Consts& c, int block, bool single) {
