@@ -415,7 +415,7 @@ struct DiffArgs {
 };
 
 __device__ __forceinline__ float4 load_command(const float* act, size_t D, int t, int d) {
-    return __ldg(reinterpret_cast<const float4*>(act + (size_t)t * D * 4) + d);
+    return reinterpret_cast<const float4*>(act + (size_t)t * D * 4)[d];
 }
 
 __device__ __forceinline__ void command4(const Consts& c, const float4 a, float fh[4], float u[4], float msk[4]) {
@@ -442,6 +442,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
     const bool act = lane < N;
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
+    await_previous();
     const bool ahead = (c.flags & QS_F_MOTOR_NOISE) && c.substeps <= FWD_SUB;
     float4* sp = sm4;            // [nb] positions; then [3][nb] velocities of the collision pass
     float* nbase = sm + 7 * nb;  // [2][FWD_SUB][4][nb] motor normals
@@ -486,6 +487,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
             L += dx * dx + dy * dy + dz * dz + 1e-3f * (fh[0] * fh[0] + fh[1] * fh[1] + fh[2] * fh[2] + fh[3] * fh[3]);
         }
     }
+    launch_next();
     if (act) {
         a.loss[d] = L;
         if (!finite_state(s)) atomicOr(dv.status, 1);
@@ -522,6 +524,7 @@ __global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_d
     const bool act = lane < N;
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
+    await_previous();
     float4* sp = sm4 + grp * nb;  // [nb] positions of the group
     float* sla = sm + 8 * nb;       // [3][nb] lambda of the acceleration (group 1)
     float* fin = sm + 11 * nb;      // [2][7][nb] position and motor noise at the end of a recomputed segment
@@ -631,6 +634,7 @@ __global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_d
         }
         __syncthreads();  // hand over: buffer it & 1 recomputed; buffer (it - 1) & 1 free again
     }
+    launch_next();
     if (grp == 1 && act) {
         float* gx = a.grad_x0 + (size_t)d * QS_STATE_DIM;
         for (int k = 0; k < 3; ++k) gx[k] = lx[k];
@@ -1195,6 +1199,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
     const bool act = lane < N;
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
+    await_previous();
     const bool coll = (c.flags & QS_F_COLLISIONS) != 0;
     const bool ahead = (c.flags & QS_F_MOTOR_NOISE) && c.substeps <= FWD_SUB;
     float4* sp = sm4;            // [nb] positions; then [3][nb] velocities of the collision pass
@@ -1245,6 +1250,7 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
             L += dx * dx + dy * dy + dz * dz + 1e-3f * (fh[0] * fh[0] + fh[1] * fh[1] + fh[2] * fh[2] + fh[3] * fh[3]);
         }
     }
+    launch_next();
     if (act) {
         a.loss[d] = L;
         if (!finite_state(s)) atomicOr(dv.status, 1);
@@ -1269,6 +1275,7 @@ __global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_d
     const bool act = lane < N;
     const int d = d0 + lane, sbase = slot * W;
     const size_t D = dv.D;
+    await_previous();
     const bool coll = (c.flags & QS_F_COLLISIONS) != 0;
     float4* sp = sm4 + grp * nb;         // [nb] positions of the group
     float* sv = sm + (8 + grp * 3) * nb; // [3][nb] velocities of the group
@@ -1392,6 +1399,7 @@ __global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_d
         }
         __syncthreads();  // hand over: buffer it & 1 recomputed; buffer (it - 1) & 1 free again
     }
+    launch_next();
     if (grp == 1 && act) {
         float* gx = a.grad_x0 + (size_t)d * QS_STATE_DIM;
         for (int k = 0; k < 3; ++k) gx[k] = lx[k];
@@ -1445,12 +1453,11 @@ cudaError_t launch_diff(int backward, const Consts& c, const Dev& dv, const Tile
         const auto k = smooth ? (dense ? k_diff_bwd<true> : k_diff_bwd<false>)
                        : et   ? (dense ? k_diffd_bwd<true, true> : k_diffd_bwd<true, false>)
                               : (dense ? k_diffd_bwd<false, true> : k_diffd_bwd<false, false>);
-        k<<<n_tiles, 2 * block, smem2, st>>>(c, dv, tiles, perm, a);
+        return launch_overlapped(k, n_tiles, 2 * block, smem2, st, c, dv, tiles, perm, a);
     } else {
         const auto k = smooth ? k_diff_fwd : et ? k_diffd_fwd<true> : k_diffd_fwd<false>;
-        k<<<n_tiles, 2 * block, smem, st>>>(c, dv, tiles, perm, a);
+        return launch_overlapped(k, n_tiles, 2 * block, smem, st, c, dv, tiles, perm, a);
     }
-    return cudaGetLastError();
 }
 
 }  // namespace qsk

@@ -13,6 +13,19 @@
 
 namespace qsk {
 
+// ---------------------------------------------------------------- launch overlap
+// The step and rollout kernels are launched with programmatic stream
+// serialisation (launch_overlapped): a kernel lets the stream's next one be
+// brought onto the device once all its own CTAs are there (launch_next), and
+// one brought on early waits, before its first access to anything an earlier
+// kernel may write, until every earlier kernel has completed and its writes
+// are visible (await_previous). Only the launch itself and the CTA's start
+// overlap. Both do nothing in a kernel launched the ordinary way. Loads of what
+// an earlier kernel may write are ordinary ones, never through the read-only
+// path (__ldg), whose data may not change while a kernel is on the device.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void await_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ---------------------------------------------------------------- Philox4x32-10
 __device__ __forceinline__ uint4 philox(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t k0, uint32_t k1) {
     uint32_t x0 = c0, x1 = c1, x2 = c2, x3 = 0u;
@@ -198,15 +211,15 @@ __device__ __forceinline__ void derive(const Consts& c, const float p7[QS_PARAM_
 // The 7 planes a step reads (m, inertia diagonal, arm, f_max, alpha_lag: 28 B
 // per env); the rest is formed by complete_prm(). t2w and tau_m enter only
 // through f_max and alpha_lag and are not loaded.
-__device__ __forceinline__ Prm load_prm(const Consts& c, const float* __restrict__ prm, int E, int e) {
+__device__ __forceinline__ Prm load_prm(const Consts& c, const float* prm, int E, int e) {
     Prm p;
-    p.m = __ldg(prm + P_M * E + e);
-    p.ixx = __ldg(prm + P_IXX * E + e);
-    p.iyy = __ldg(prm + P_IYY * E + e);
-    p.izz = __ldg(prm + P_IZZ * E + e);
-    p.arm = __ldg(prm + P_ARM * E + e);
-    p.fmax = __ldg(prm + P_FMAX * E + e);
-    p.alag = __ldg(prm + P_ALAG * E + e);
+    p.m = prm[P_M * E + e];
+    p.ixx = prm[P_IXX * E + e];
+    p.iyy = prm[P_IYY * E + e];
+    p.izz = prm[P_IZZ * E + e];
+    p.arm = prm[P_ARM * E + e];
+    p.fmax = prm[P_FMAX * E + e];
+    p.alag = prm[P_ALAG * E + e];
     p.t2w = 0.f;
     p.tau = 0.f;
     complete_prm(c, p);

@@ -125,12 +125,32 @@ struct RolloutIO {
     bool bulk;         // obs is device memory (rows may leave by bulk asynchronous copies)
 };
 
+#ifdef __CUDACC__
+// Launches kernel so that it may be brought onto the device while the stream's
+// previous kernel ends (launch_next(), await_previous() in qs_device.cuh).
+template <class... P, class... A>
+cudaError_t launch_overlapped(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+#endif
+
 // kernels (qs_step.cu)
 cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, const Tile* tiles, const int* perm,
                         const StepIO& io, int observe_only, cudaStream_t s);
 // Persistent launch over n_tiles tiles (any classes) of `block` threads;
 // steps t0 .. t0+nsteps-1 of the io buffers. grid <= 0: one CTA per tile.
 // single: every env of the handle holds one drone (the single-drone instance).
+// *counter is 0 before and after the launch.
 cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int block, const int* perm,
                            int* counter, const RolloutIO& io, int t0, int nsteps, int grid, bool single,
                            cudaStream_t s);

@@ -439,12 +439,20 @@ __device__ __forceinline__ SlotMap map_slot(const Dev& dv, const Tile& tile, con
 
 // W = 1 (one drone per env) is HBM-bound at scale: capping it at 80 registers
 // (a few dozen bytes of spills to L1) keeps 12 CTAs of 64 threads per SM in
-// flight instead of 9, +18% at 1M envs.
-template <int W, bool EXT>
-__global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
+// flight instead of 9, +18% at 1M envs. Swarms of up to 32 keep 96 (10 CTAs of
+// 64 threads instead of 8; 131,072 x 8, K = 6, 191 -> 173 us a step, 32,768 x 8
+// 62 -> 56), wider ones, whose pair pass is most of the step, what they need
+// (64 x 256: 9.5 against 10.0 us). OVERLAP: launched overlapped with the
+// stream's previous kernel, for up to STEP_OVERLAP_WAVES waves (65,536 single
+// drones 10.3 -> 8.0 us a step, 262,144 28.7 -> 28.3); past them every CTA's
+// wait costs more than the launch (1,048,576: 83.2 -> 87.9 us).
+constexpr int STEP_OVERLAP_WAVES = 2;
+template <int W, bool EXT, bool OVERLAP = true>
+__global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                     const int* __restrict__ perm, const StepIO io, const int observe_only) {
     extern __shared__ float4 sm[];
     const SlotMap m = map_slot(dv, tile_at(dv, tiles, blockIdx.x, blockDim.x), perm, W);
+    if (OVERLAP) await_previous();
     Drone s;
     EnvRegs er;
     uint32_t ev = 0;
@@ -452,7 +460,7 @@ __global__ void __launch_bounds__(MAX_BLOCK, (W == 1 ? 3 : 1)) k_step(const Cons
         load_drone(s, dv.st, dv.D, m.d);
         load_env<EXT>(er, c, dv, m.e);
     }
-    const float4 a = (m.act && !observe_only) ? __ldg(reinterpret_cast<const float4*>(io.act) + m.d)
+    const float4 a = (m.act && !observe_only) ? reinterpret_cast<const float4*>(io.act)[m.d]
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
     float gv[GOAL_VALUES];
     GoalCache gc{gv, GOAL_FIXED, 0, -1};
@@ -483,14 +491,14 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
     const float4* act4 = reinterpret_cast<const float4*>(io.act) + m.d;
     // the commands of step t + 1 are loaded while step t computes, so their
     // HBM latency leaves each step's dependent chain
-    float4 a_next = m.act ? __ldg(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 a_next = m.act ? *(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
     float* goals = reinterpret_cast<float*>(sm + 2 * SMEM_PLANES / 4 * blockDim.x);  // the general instance's goal values
     GoalCache gc{goals + GOAL_STRIDE * threadIdx.x, GOAL_FIXED, 0, -1};
     const RowMap rm = W1 ? RowMap() : map_rows(m.act, m.d, W, c.obs_dim);
     float* rows = goals + (EXT ? GOAL_STRIDE * blockDim.x : 0) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
     for (int t = t0; t < t0 + nsteps; ++t) {
         const float4 a = a_next;
-        if (m.act && t + 1 < t0 + nsteps) a_next = __ldg(act4 + (size_t)(t + 1) * D);
+        if (m.act && t + 1 < t0 + nsteps) a_next = *(act4 + (size_t)(t + 1) * D);
         float4* sp = sm + ((t - t0) & 1) * (SMEM_PLANES / 4) * blockDim.x;
         step_body<EXT, !W1>(W, c, dv, s, er, ev, sp, reinterpret_cast<float*>(sp + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a,
                        io.obs ? io.obs + (size_t)t * D * c.obs_dim : nullptr, io.rew ? io.rew + (size_t)t * D : nullptr,
@@ -504,8 +512,10 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
     }
 }
 
-// Persistent rollout: CTAs take tiles from *counter (zeroed before the launch)
-// until none is left. Tiles are ordered costliest first. The W1 instance
+// Persistent rollout: CTAs take tiles from *counter until none is left; every
+// CTA draws one number past the tiles, and the last of those puts the counter
+// back to zero for the next launch (a memset before each launch cost a launch
+// of its own). Tiles are ordered costliest first. The W1 instance
 // (EXT = false only) serves handles whose envs all hold one drone: 107
 // registers instead of 121 and no untaken swarm code in the step loop (with
 // the smooth contacts compiled out of the EXT = false instances, batched
@@ -518,12 +528,19 @@ __global__ void __launch_bounds__(MAX_BLOCK, 2) k_rollout(const Consts c, const 
                                                        const int nsteps) {
     extern __shared__ float4 sm[];
     __shared__ int s_next;
+    await_previous();
     for (;;) {
-        if (threadIdx.x == 0) s_next = atomicAdd(counter, 1);
+        if (threadIdx.x == 0) {
+            s_next = atomicAdd(counter, 1);
+            if (s_next == n_tiles + (int)gridDim.x - 1) *counter = 0;
+        }
         __syncthreads();
         const int ti = s_next;
         __syncthreads();  // everyone has read s_next before thread 0 overwrites it
-        if (ti >= n_tiles) return;
+        if (ti >= n_tiles) {
+            launch_next();
+            return;
+        }
         rollout_tile<EXT, W1>(c, dv, tile_at(dv, tiles, ti, blockDim.x), perm, sm, io, t0, nsteps);
     }
 }
@@ -858,6 +875,7 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
     __shared__ WsShared<1> sh;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, 32);
     const WsMap m = ws_map<1>(dv, tile, perm);
+    await_previous();
     if (threadIdx.x >= 32) {
         // ---------------- noise warp
         const uint32_t tick = m.act ? dv.tick[m.e] : 0u;  // warp 0 writes it only after B2
@@ -866,6 +884,7 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
         float ex[3] = {0.f, 0.f, 0.f}, evv[3] = {0.f, 0.f, 0.f}, ew[3] = {0.f, 0.f, 0.f};
         if (m.act && io.obs && (c.flags & QS_F_OBS_NOISE)) obs_noise(c, tick, m.d, 0u, ex, evv, ew);
         __syncthreads();  // B2
+        launch_next();
         if (io.obs) ws_store_obs<1>(c, dv, tile, perm, sh, m, 0, io.obs, ex, evv, ew);
         return;
     }
@@ -877,7 +896,7 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
     if (m.act) {
         load_drone(s, dv.st, dv.D, m.d);
         load_env<EXT>(er, c, dv, m.e);
-        a = __ldg(reinterpret_cast<const float4*>(io.act) + m.d);
+        a = reinterpret_cast<const float4*>(io.act)[m.d];
     }
     GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
     ws_dynamics_step<EXT, 1, false>(c, dv, sh, m, s, er, ev, a, 0, io.rew, io.done, gc);
@@ -906,6 +925,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
     const Tile tile = tile_at(dv, tiles, blockIdx.x, 32 * P);
     const WsMap m = ws_map<P>(dv, tile, perm);
     const size_t D = dv.D, E = dv.E;
+    await_previous();
     if (threadIdx.x >= 32 * P) {
         // ---------------- noise side; the env's Philox counter advances by one per step
         // Step t's observation rows and reward are finished during step t + 1's
@@ -956,6 +976,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
             }
             __syncthreads();  // B2 of step t
         }
+        launch_next();
         if (nsteps > 0) finish(nsteps - 1);  // after the last B2
         return;
     }
@@ -968,11 +989,11 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
         load_env<EXT>(er, c, dv, m.e);
     }
     const float4* act4 = reinterpret_cast<const float4*>(io.act) + m.d;
-    float4 a_next = m.act ? __ldg(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 a_next = m.act ? *(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
     GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
     for (int t = 0; t < nsteps; ++t) {
         const float4 a = a_next;
-        if (m.act && t + 1 < nsteps) a_next = __ldg(act4 + (size_t)(t0 + t + 1) * D);
+        if (m.act && t + 1 < nsteps) a_next = *(act4 + (size_t)(t0 + t + 1) * D);
         ws_dynamics_step<EXT, P, true>(c, dv, sh, m, s, er, ev, a, t & 1,
                                  io.rew ? io.rew + (size_t)(t0 + t) * D : nullptr,
                                  io.done ? io.done + (size_t)(t0 + t) * E : nullptr, gc, t == 0 || m.W > 1);
@@ -1184,34 +1205,44 @@ int rollout_ws_resident_ctas(const Consts& c, int P) {
     return occ * n_sm;
 }
 
+// CTAs of `block` threads of the single-drone step (80 registers) in a wave.
+int step_wave(int block) {
+    int dev = 0, n_sm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    return n_sm * (768 / block);
+}
+
 template <bool EXT>
 cudaError_t launch_k_step(const Consts& c, const Dev& dv, const ClassPlan& cp, const Tile* t, const int* perm,
                           const StepIO& io, int observe_only, size_t smem, cudaStream_t st) {
+    const auto k = [&](auto kernel) {
+        return launch_overlapped(kernel, cp.n_tiles, cp.block, smem, st, c, dv, t, perm, io, observe_only);
+    };
     switch (cp.W) {
-        case 1: k_step<1, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 2: k_step<2, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 4: k_step<4, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 8: k_step<8, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 16: k_step<16, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 32: k_step<32, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 64: k_step<64, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
-        case 128: k_step<128, EXT><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only); break;
+        case 1: {
+            if (cp.n_tiles <= STEP_OVERLAP_WAVES * step_wave(cp.block)) return k(k_step<1, EXT>);
+            k_step<1, EXT, false><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only);
+            return cudaGetLastError();
+        }
+        case 2: return k(k_step<2, EXT>);
+        case 4: return k(k_step<4, EXT>);
+        case 8: return k(k_step<8, EXT>);
+        case 16: return k(k_step<16, EXT>);
+        case 32: return k(k_step<32, EXT>);
+        case 64: return k(k_step<64, EXT>);
+        case 128: return k(k_step<128, EXT>);
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, const Tile* tiles, const int* perm,
                         const StepIO& io, int observe_only, cudaStream_t st) {
     if (cp.n_tiles == 0) return cudaSuccess;
     const bool ext = extended(c);
-    if (cp.ws && !observe_only) {
-        if (ext)
-            k_step_ws<true><<<cp.n_tiles, 64, 0, st>>>(c, dv, tiles + cp.tile_off, perm, io);
-        else
-            k_step_ws<false><<<cp.n_tiles, 64, 0, st>>>(c, dv, tiles + cp.tile_off, perm, io);
-        return cudaGetLastError();
-    }
+    if (cp.ws && !observe_only)
+        return launch_overlapped(ext ? k_step_ws<true> : k_step_ws<false>, cp.n_tiles, 64, 0, st, c, dv, tiles + cp.tile_off,
+                                 perm, io);
     const size_t smem = (cp.W > 1) ? sizeof(float) * SMEM_PLANES * cp.block : 0;
     const Tile* t = tiles + cp.tile_off;
     return ext ? launch_k_step<true>(c, dv, cp, t, perm, io, observe_only, smem, st)
@@ -1254,39 +1285,22 @@ cudaError_t launch_rollout_ws(const Consts& c, const Dev& dv, const Tile* tiles,
                               const RolloutIO& io, int t0, int nsteps, cudaStream_t st) {
     if (n_tiles == 0) return cudaSuccess;
     const bool ext = extended(c);
-    if (P == 1) {
-        if (ext)
-            k_rollout_ws<true, 1><<<n_tiles, 64, 0, st>>>(c, dv, tiles, perm, io, t0, nsteps);
-        else
-            k_rollout_ws<false, 1><<<n_tiles, 64, 0, st>>>(c, dv, tiles, perm, io, t0, nsteps);
-    } else if (P == 2) {
-        if (ext)
-            k_rollout_ws<true, 2><<<n_tiles, 128, 0, st>>>(c, dv, tiles, perm, io, t0, nsteps);
-        else
-            k_rollout_ws<false, 2><<<n_tiles, 128, 0, st>>>(c, dv, tiles, perm, io, t0, nsteps);
-    } else {
-        return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    if (P != 1 && P != 2) return cudaErrorInvalidValue;
+    const auto k = P == 1 ? (ext ? k_rollout_ws<true, 1> : k_rollout_ws<false, 1>)
+                          : (ext ? k_rollout_ws<true, 2> : k_rollout_ws<false, 2>);
+    return launch_overlapped(k, n_tiles, 64 * P, 0, st, c, dv, tiles, perm, io, t0, nsteps);
 }
 
 cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int block, const int* perm,
                            int* counter, const RolloutIO& io, int t0, int nsteps, int grid, bool single,
                            cudaStream_t st) {
-    cudaError_t e = cudaMemsetAsync(counter, 0, sizeof(int), st);
-    if (e != cudaSuccess) return e;
     const size_t smem = rollout_smem(c, block, single);
-    e = allow_smem(rollout_kernel(extended(c), single), smem);
+    const cudaError_t e = allow_smem(rollout_kernel(extended(c), single), smem);
     if (e != cudaSuccess) return e;
     const int g = grid > 0 ? grid : n_tiles;
     const int grid_n = g < n_tiles ? g : n_tiles;
-    if (extended(c))
-        k_rollout<true, false><<<grid_n, block, smem, st>>>(c, dv, tiles, n_tiles, perm, counter, io, t0, nsteps);
-    else if (single)
-        k_rollout<false, true><<<grid_n, block, smem, st>>>(c, dv, tiles, n_tiles, perm, counter, io, t0, nsteps);
-    else
-        k_rollout<false, false><<<grid_n, block, smem, st>>>(c, dv, tiles, n_tiles, perm, counter, io, t0, nsteps);
-    return cudaGetLastError();
+    const auto k = extended(c) ? k_rollout<true, false> : single ? k_rollout<false, true> : k_rollout<false, false>;
+    return launch_overlapped(k, grid_n, block, smem, st, c, dv, tiles, n_tiles, perm, counter, io, t0, nsteps);
 }
 
 }  // namespace qsk
