@@ -542,6 +542,7 @@ qs_status qs_create(const qs_config* cfg, void* cuda_stream, qs_env** out) {
             const int per = std::max(1, 32 / h->plan[ci].W);
             ws_ctas += (h->class_slots[ci] + per - 1) / per;
         }
+        if (maxW == 1) h->rollout_block = 32;  // 1,048,576 drones, 32 steps: 32 / 64 / 128 threads 1586 / 1618 / 1632 us
         const bool ext = (h->c.scn_mask & ~1u) != 0 || (h->c.flags & QS_F_DOWNWASH) != 0;
         if (maxW <= 32 && (!ext || h->plan.size() == 1) && ws_ctas <= rollout_ws_resident_ctas(h->c, 1) &&
             (maxW <= 16 || ws_ctas <= 5L * n_sm))

@@ -520,9 +520,12 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
 // registers instead of 121 and no untaken swarm code in the step loop (with
 // the smooth contacts compiled out of the EXT = false instances, batched
 // 1,048,576 single-drone envs went from 1.75e10 to 1.90e10 quadrotor-steps/s,
-// each change about half of it).
+// each change about half of it). Held to 104 registers it fits in 96 without a
+// spill, five warps a scheduler instead of four (1,048,576 drones, 32 steps,
+// 1687 -> 1632 us, in 32-thread CTAs 1593; at 88 registers 1644). Swarms spill
+// below 128 (16,384 x 8, 64 steps: 128 registers 746 us, 112 799, 160 901).
 template <bool EXT, bool W1>
-__global__ void __launch_bounds__(MAX_BLOCK, 2) k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
+__global__ void __maxnreg__(W1 ? 104 : 128) k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                        const int n_tiles, const int* __restrict__ perm,
                                                        int* __restrict__ counter, const RolloutIO io, const int t0,
                                                        const int nsteps) {
