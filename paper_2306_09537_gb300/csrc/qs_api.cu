@@ -175,10 +175,7 @@ void build_tiles(qs_env* h, std::vector<Tile>& tiles) {
         cp.tile_off = (int)tiles.size();
         cp.n_tiles = 0;
         for (int s = 0; s < h->class_slots[ci]; s += per) {
-            const int first = h->class_first_slot[ci] + s, count = std::min(per, h->class_slots[ci] - s);
-            int contig = 1;
-            for (int i = 1; i < count; ++i) contig &= h->perm_h[first + i] == h->perm_h[first] + i;
-            tiles.push_back(Tile{first, count, cp.W, contig});
+            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), cp.W, 0});
             ++cp.n_tiles;
         }
     }
@@ -208,12 +205,8 @@ void build_ws_tiles(qs_env* h, std::vector<Tile>& tiles) {
     if (!h->ws_p) return;
     for (size_t ci = 0; ci < h->plan.size(); ++ci) {
         const int W = h->plan[ci].W, per = 32 * h->ws_p / W;
-        for (int s = 0; s < h->class_slots[ci]; s += per) {
-            const int first = h->class_first_slot[ci] + s, count = std::min(per, h->class_slots[ci] - s);
-            int contig = 1;
-            for (int i = 1; i < count; ++i) contig &= h->perm_h[first + i] == h->perm_h[first] + i;
-            tiles.push_back(Tile{first, count, W, contig});
-        }
+        for (int s = 0; s < h->class_slots[ci]; s += per)
+            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), W, 0});
     }
 }
 
@@ -359,7 +352,7 @@ bool device_memory(const void* p) {
 // the per-class kernels; measured on GB300 with sizes 1..64: 4096 envs 90.8
 // -> 35.5 us, 65,536 envs 271 -> 207 us); one class keeps its per-call kernel.
 qs_status do_step(qs_env* h, const float* act, float* obs, float* rew, uint8_t* done) {
-    if (h->plan.size() > 1) return enqueue_rollout(h, 1, RolloutIO{act, obs, rew, done, device_memory(obs)});
+    if (h->plan.size() > 1) return enqueue_rollout(h, 1, RolloutIO{act, obs, rew, done, false});
     StepIO io{act, obs, rew, done};
     for (const ClassPlan& cp : h->plan) {
         cudaError_t e = launch_step(h->c, h->dv, cp, h->d_tiles, h->d_perm, io, 0, h->stream);

@@ -96,7 +96,7 @@ struct Tile {
     int first;  // first slot (index into perm)
     int count;  // slots in this tile
     int W;      // width class of its slots
-    int pad;    // 1: the tile's envs are consecutive, so its drones are contiguous
+    int pad;
 };
 
 struct ClassPlan {

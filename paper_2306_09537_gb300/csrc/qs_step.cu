@@ -207,7 +207,8 @@ struct RowMap {
     int d0, n;   // first drone and rows of the lane's block
     int off;     // the block's floats in the warp's buffer start here (a multiple of 4)
     int rank;    // row of this lane's drone in it
-    bool lead;   // this lane copies the block
+    int gl, gs;  // this lane's place among the gs lanes that share the block
+    bool lead;   // the lane that hands the block over
 };
 
 __device__ __forceinline__ RowMap map_rows(bool act, int d, int W, int od) {
@@ -217,11 +218,11 @@ __device__ __forceinline__ RowMap map_rows(bool act, int d, int W, int od) {
     const int f0 = __shfl_sync(0xffffffffu, d - rank, lead);
     const bool one = __all_sync(0xffffffffu, !act || d - rank == f0);
     if (one) {
-        r = RowMap{f0, __popc(am), 0, rank, act && ln == lead};
+        r = RowMap{f0, __popc(am), 0, rank, ln, 32, act && ln == lead};
     } else {  // slots of one warp: W <= 16
         const int slot = ln / W, l0 = slot * W;
         r = RowMap{d - (ln - l0), __popc(am >> l0 & ((1u << W) - 1u)), slot * (((W * od + 3) & ~3) + 4), ln - l0,
-                   act && ln == l0};
+                   ln - l0, W, act && ln == l0};
     }
     return r;
 }
@@ -237,36 +238,32 @@ __device__ __forceinline__ void rows_free(const RowMap& r) {
     __syncwarp();
 }
 
-// Starts the copies of the warp's blocks (every lane calls it), or without
-// bulk (a destination in host memory) stores each lane's row.
-__device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, float* __restrict__ obs, int od, bool act,
-                                          bool bulk) {
-    float* dst = obs + (size_t)r.d0 * od;
+// Sends the warp's blocks on their way (every lane calls it): bulk copies, or
+// without bulk (destinations that may lie in host memory) stores by the lanes
+// that share a block, side by side.
+__device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, float* __restrict__ obs, int od, bool bulk) {
     const int sh = row_shift(r, obs, od);
+    const int n = r.n * od - sh, m = n & ~3;  // floats past the 8 bytes before the units
     const float* src = rows + r.off + sh;
-    if (!bulk) {
-        const float2* s2 = reinterpret_cast<const float2*>(src + r.rank * od);
-        float2* d2 = reinterpret_cast<float2*>(dst + (size_t)r.rank * od);
-        if (act)
-            for (int i = 0; i < od / 2; ++i) d2[i] = s2[i];
-        return;
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    float* dst = obs + (size_t)r.d0 * od;
+    if (bulk) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncwarp();
+    if (!bulk) {
+        const float4* s4 = reinterpret_cast<const float4*>(src + sh);
+        float4* d4 = reinterpret_cast<float4*>(dst + sh);
+        for (int i = r.gl; i < (m >> 2); i += r.gs) d4[i] = s4[i];
+    }
     if (r.lead) {
-        const int n = r.n * od - sh, m = n & ~3;  // floats past the 8 bytes before the units
         if (sh) *reinterpret_cast<float2*>(dst) = *reinterpret_cast<const float2*>(src);
         if (n & 2) *reinterpret_cast<float2*>(dst + sh + m) = *reinterpret_cast<const float2*>(src + sh + m);
-        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(dst + sh),
-                     "r"((uint32_t)__cvta_generic_to_shared(src + sh)), "r"(4 * m)
-                     : "memory");
+        if (bulk)
+            asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n\tcp.async.bulk.commit_group;" ::"l"(
+                             dst + sh),
+                         "r"((uint32_t)__cvta_generic_to_shared(src + sh)), "r"(4 * m)
+                         : "memory");
     }
 }
 
-// One control step of the slot's drones. All threads of the CTA call it (the
-// pair pass synchronises the CTA); `act` marks threads that carry a drone.
-// Outputs for this step: obs/rew rows of drone d, done[e] (lane 0). W is
-// uniform over the CTA; a compile-time W folds away after inlining.
 // ROWS: the observation rows go through shared memory (the rollout), else each
 // lane stores its own. Swarm rollouts take the former (4096 uneven swarms, 32
 // steps, 358 -> 299 us; 256 x 128, 16 steps, 203 -> 183 us); single drones keep
@@ -398,7 +395,7 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
             }
         }
     }
-    if (ROWS && obs) send_rows(rm, rows, obs, c.obs_dim, act, bulk);
+    if (ROWS && obs) send_rows(rm, rows, obs, c.obs_dim, bulk);
     if (!act || observe_only) return;
 
     if ((c.flags & QS_F_RECORD_KNN) && dv.knn) {
@@ -554,33 +551,38 @@ __global__ void __maxnreg__(W1 ? 104 : 128) k_rollout(const Consts c, const Dev 
 // through the substeps and the pair pass. Warps P .. 2P-1 (noise) draw the
 // motor-noise normals of the first WS_SUB substeps into shared memory ahead of
 // the dynamics, then the observation noise while the dynamics run, and finally
-// assemble the observation rows of the CTA's drones in shared memory and store
-// them; when the CTA's drones are contiguous in memory the rows form one block
-// written with 16-byte stores. The two sides meet at two CTA barriers: after
+// put the observation rows of their drones together in shared memory and send
+// them (RowMap). The two sides meet at two CTA barriers: after
 // the motor normals (B1) and after the dynamics warps publish the final states
 // (B2). This takes the Philox and Box-Muller work off each drone's dependent
 // chain. With P = 2 (swarms of 33..64) the dynamics warps also meet at named
 // barrier 1 between staging and reading each other's positions, and the noise
-// warps at named barrier 2 before storing the block of rows.
+// warps at named barrier 2 between writing and reading swap keys.
 constexpr int WS_SUB = 4;
-constexpr int WS_OBS_MAX = 18 + 6 * QS_MAX_K;
 
+// What the two sides exchange, one entry a drone lane, in 8- and 16-byte words
+// (a warp's load or store of one is as many instructions as its words). The
+// noise side's observation rows follow in dynamic shared memory (ws_smem).
 template <int P>
 struct WsShared {
-    float nrm[2][WS_SUB][4][32 * P];  // motor-noise normals [buffer][substep][rotor][drone lane]
-    // the published end of a step, [buffer] by step parity:
-    float st[2][18][32 * P];          // x v R w of each drone lane after the step (post-collision)
-    float g[2][3][32 * P];            // goal of each lane's drone
-    NbrList nb[2][32 * P];            // CTA drone lanes of the neighbours
-    int keff[2][32 * P];
-    float rin[2][9][32 * P];          // reward inputs: command f^ (4), previous command (4), proximity radius
-    uint32_t ev[2][32 * P];           // event bits
-    float4 sp[32 * P];                // pair-pass staging: positions
-    float sv[3][32 * P];              //                    velocities
-    uint32_t key[32 * P];             // swap keys
-    float gv[32 * P][GOAL_STRIDE];    // goal values of each lane's drone (GoalCache)
-    float rows[32 * P * WS_OBS_MAX];
+    float4 nrm[2][WS_SUB][32 * P];  // motor-noise normals of the four rotors [buffer][substep]
+    // the published end of a step (post-collision), [buffer] by step parity:
+    float4 px[2][32 * P];           // x, y, z, v_x
+    float2 vyz[2][32 * P];          // v_y, v_z
+    float4 rw[2][3][32 * P];        // R row-major, w
+    float4 gk[2][32 * P];           // goal, number of neighbours (bits)
+    NbrList nb[2][32 * P];          // CTA drone lanes of the neighbours
+    float4 fh[2][32 * P];           // reward inputs: command f^,
+    float4 fp[2][32 * P];           //   previous command,
+    float2 pe[2][32 * P];           //   proximity radius, event bits
+    float4 sp[32 * P];              // pair-pass staging: positions
+    float sv[3][32 * P];            //                    velocities
+    uint32_t key[32 * P];           // swap keys
+    float gv[32 * P][GOAL_STRIDE];  // goal values of each lane's drone (GoalCache)
 };
+
+// Dynamic shared memory of a warp-specialised CTA: the noise side's rows.
+inline size_t ws_smem(const Consts& c, int P) { return sizeof(float) * 32 * P * (c.obs_dim + ROW_PAD); }
 
 // Barrier among the P warps of one side (id 1: dynamics, id 2: noise); one
 // warp only needs its own lanes converged.
@@ -626,74 +628,7 @@ __device__ __forceinline__ void ws_motor_normals(const Consts& c, WsShared<P>& s
     for (int sub = 0; sub < nahead; ++sub) {
         float n[4];
         motor_normals(c, tick, m.d, sub, n);
-        sh.nrm[nb][sub][0][m.L] = n[0];
-        sh.nrm[nb][sub][1][m.L] = n[1];
-        sh.nrm[nb][sub][2][m.L] = n[2];
-        sh.nrm[nb][sub][3][m.L] = n[3];
-    }
-}
-
-// Noise side, after B2: the observation rows of the CTA's drones from the
-// published post-step states plus sensor noise, assembled in shared memory and
-// stored to obs; when the CTA's drones are contiguous the rows form one block
-// written with 16-byte stores.
-template <int P>
-__device__ __forceinline__ void ws_store_obs(const Consts& c, const Dev& dv, const Tile& tile,
-                                             const int* __restrict__ perm, WsShared<P>& sh, const WsMap& m, int b,
-                                             float* __restrict__ obs, const float ex[3], const float evv[3],
-                                             const float ew[3]) {
-    const int od = c.obs_dim, K = c.K, L = m.L;
-    const float(&st)[18][32 * P] = sh.st[b];
-    const bool contig = tile.pad != 0 &&
-                        qs_check(dv.status, tile.first >= 0 && tile.count >= 1 && tile.first + tile.count <= dv.E);
-    const int d_first = contig ? env_first(dv, slot_env(dv, perm, tile.first)) : 0;
-    const int ridx = contig ? m.d - d_first : L;
-    if (m.act) {
-        float* row = sh.rows + ridx * od;
-        row[0] = st[0][L] - sh.g[b][0][L] + ex[0];
-        row[1] = st[1][L] - sh.g[b][1][L] + ex[1];
-        row[2] = st[2][L] - sh.g[b][2][L] + ex[2];
-        row[3] = st[3][L] + evv[0];
-        row[4] = st[4][L] + evv[1];
-        row[5] = st[5][L] + evv[2];
-        for (int k = 6; k < 15; ++k) row[k] = st[k][L];
-        row[15] = st[15][L] + ew[0];
-        row[16] = st[16][L] + ew[1];
-        row[17] = st[17][L] + ew[2];
-        const int ke = sh.keff[b][L];
-        const NbrList nb = sh.nb[b][L];
-        for (int k = 0; k < K; ++k) {
-            float* on = row + 18 + 6 * k;
-            if (k < ke) {
-                const int j = nbr_at(nb, k);
-                for (int q = 0; q < 6; ++q) on[q] = st[q][j] - st[q][L];
-            } else {
-                for (int q = 0; q < 6; ++q) on[q] = 0.f;
-            }
-        }
-    }
-    side_sync<P>(2);
-    const int e_last = contig ? slot_env(dv, perm, tile.first + tile.count - 1) : 0;
-    const int d_end = contig ? env_first(dv, e_last + 1) : 0;
-    if (contig && qs_check(dv.status, d_first >= 0 && d_end <= dv.D && d_end - d_first <= 32 * P)) {
-        const int n_floats = (d_end - d_first) * od;
-        float* dst = obs + (size_t)d_first * od;
-        if (((uintptr_t)dst & 15u) == 0) {
-            const int n4 = n_floats >> 2;
-            const float4* src4 = reinterpret_cast<const float4*>(sh.rows);
-            float4* dst4 = reinterpret_cast<float4*>(dst);
-            for (int i = L; i < n4; i += 32 * P) dst4[i] = src4[i];
-            for (int i = (n4 << 2) + L; i < n_floats; i += 32 * P) dst[i] = sh.rows[i];
-        } else {
-            const int n2 = n_floats >> 1;  // obs rows hold an even number of floats
-            const float2* src2 = reinterpret_cast<const float2*>(sh.rows);
-            float2* dst2 = reinterpret_cast<float2*>(dst);
-            for (int i = L; i < n2; i += 32 * P) dst2[i] = src2[i];
-        }
-    } else if (m.act && !contig) {
-        const float2* src2 = reinterpret_cast<const float2*>(sh.rows + ridx * od);
-        float2* dst2 = reinterpret_cast<float2*>(obs + (size_t)m.d * od);
-        for (int i = 0; i < od / 2; ++i) dst2[i] = src2[i];
+        sh.nrm[nb][sub][m.L] = make_float4(n[0], n[1], n[2], n[3]);
     }
 }
 
@@ -762,8 +697,8 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
             side_sync<P>(1);
             if (act) {
                 if (mnoise && sub < nahead) {
-                    const float n[4] = {sh.nrm[nb][sub][0][L], sh.nrm[nb][sub][1][L], sh.nrm[nb][sub][2][L],
-                                        sh.nrm[nb][sub][3][L]};
+                    const float4 q = sh.nrm[nb][sub][L];
+                    const float n[4] = {q.x, q.y, q.z, q.w};
                     ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, pacc, n);
                 } else {
                     ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, pacc);
@@ -774,8 +709,8 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         const float zero3[3] = {0.f, 0.f, 0.f};
         for (int sub = 0; sub < c.substeps; ++sub) {
             if (mnoise && sub < nahead) {
-                const float n[4] = {sh.nrm[nb][sub][0][L], sh.nrm[nb][sub][1][L], sh.nrm[nb][sub][2][L],
-                                    sh.nrm[nb][sub][3][L]};
+                const float4 q = sh.nrm[nb][sub][L];
+                const float n[4] = {q.x, q.y, q.z, q.w};
                 ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, zero3, n);
             } else {
                 ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, zero3);
@@ -809,23 +744,17 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
     float gl[3] = {er.g0, er.g1, er.g2};
     if (EXT && !DEFER && (c.scn_mask & ~1u)) ws_goal<P>(c, dv, sh, m, er.sel, er.ep + 1, gc, gl, 1);
     if (act) {  // publish the observed state (post-collision) for the noise side
-        const float v18[18] = {s.x[0], s.x[1], s.x[2], s.v[0], s.v[1], s.v[2], s.R[0], s.R[1], s.R[2],
-                               s.R[3], s.R[4], s.R[5], s.R[6], s.R[7], s.R[8], s.w[0], s.w[1], s.w[2]};
-#pragma unroll
-        for (int k = 0; k < 18; ++k) sh.st[b][k][L] = v18[k];
-        sh.g[b][0][L] = gl[0];
-        sh.g[b][1][L] = gl[1];
-        sh.g[b][2][L] = gl[2];
-        sh.keff[b][L] = W > 1 ? keff : 0;
+        sh.px[b][L] = make_float4(s.x[0], s.x[1], s.x[2], s.v[0]);
+        sh.vyz[b][L] = make_float2(s.v[1], s.v[2]);
+        sh.rw[b][0][L] = make_float4(s.R[0], s.R[1], s.R[2], s.R[3]);
+        sh.rw[b][1][L] = make_float4(s.R[4], s.R[5], s.R[6], s.R[7]);
+        sh.rw[b][2][L] = make_float4(s.R[8], s.w[0], s.w[1], s.w[2]);
+        sh.gk[b][L] = make_float4(gl[0], gl[1], gl[2], __int_as_float(W > 1 ? keff : 0));
         sh.nb[b][L] = nbrs + (NbrList)sbase * 0x0101010101010101ull;  // (fields past keff are not read)
         if (DEFER) {  // the noise side computes the reward from these
-#pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                sh.rin[b][r][L] = fh[r];
-                sh.rin[b][4 + r][L] = s.fp[r];
-            }
-            sh.rin[b][8][L] = er.p.prox;
-            sh.ev[b][L] = ev;
+            sh.fh[b][L] = make_float4(fh[0], fh[1], fh[2], fh[3]);
+            sh.fp[b][L] = make_float4(s.fp[0], s.fp[1], s.fp[2], s.fp[3]);
+            sh.pe[b][L] = make_float2(er.p.prox, __uint_as_float(ev));
         }
     }
     __syncthreads();  // B2
@@ -845,31 +774,83 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
     ev_out = ev;
 }
 
-// Noise side: the reward of the step published in buffer b (the same
-// compute_reward as the dynamics side, on the published post-step state).
-template <int P>
-__device__ __forceinline__ void ws_reward(const Consts& c, WsShared<P>& sh, const WsMap& m, int b,
-                                          float* __restrict__ rew) {
-    if (!m.act) return;
-    const int L = m.L;
+// Noise side: finishes the step published in buffer b. The observation rows
+// (with sensor noise ex, evv, ew) go to obs, and with rew the reward (the same
+// compute_reward as the dynamics side) of the lane's drone; goal(gl) replaces
+// the published single goal where scenarios are on. Every thread of the side
+// calls it. The rows took two thirds of the noise side's time, word by word:
+// 3,800 of 7,200 cycles a step for swarms of 8 at K = 6 (two CTAs an SM).
+template <int P, class Goal>
+__device__ __forceinline__ void ws_finish(const Consts& c, WsShared<P>& sh, const WsMap& m, const RowMap& rm, float* rows,
+                                          int b, float* __restrict__ obs, float* __restrict__ rew, bool bulk,
+                                          const float ex[3], const float evv[3], const float ew[3], const Goal& goal) {
+    const int L = m.L, od = c.obs_dim, K = c.K;
     Drone s;
-    for (int k = 0; k < 3; ++k) {
-        s.x[k] = sh.st[b][k][L];
-        s.v[k] = sh.st[b][3 + k][L];
-        s.w[k] = sh.st[b][15 + k][L];
+    float gl[3] = {0.f, 0.f, 0.f};
+    int keff = 0;
+    NbrList nb = 0;
+    if (m.act) {
+        const float4 a = sh.px[b][L], r0 = sh.rw[b][0][L], r1 = sh.rw[b][1][L], r2 = sh.rw[b][2][L], g = sh.gk[b][L];
+        const float2 v = sh.vyz[b][L];
+        nb = sh.nb[b][L];
+        s.x[0] = a.x; s.x[1] = a.y; s.x[2] = a.z;
+        s.v[0] = a.w; s.v[1] = v.x; s.v[2] = v.y;
+        s.R[0] = r0.x; s.R[1] = r0.y; s.R[2] = r0.z; s.R[3] = r0.w; s.R[4] = r1.x; s.R[5] = r1.y; s.R[6] = r1.z;
+        s.R[7] = r1.w; s.R[8] = r2.x;
+        s.w[0] = r2.y; s.w[1] = r2.z; s.w[2] = r2.w;
+        gl[0] = g.x; gl[1] = g.y; gl[2] = g.z;
+        keff = __float_as_int(g.w);
     }
-    for (int k = 0; k < 9; ++k) s.R[k] = sh.st[b][6 + k][L];
-    float fh[4];
-    for (int r = 0; r < 4; ++r) {
-        fh[r] = sh.rin[b][r][L];
-        s.fp[r] = sh.rin[b][4 + r][L];
+    goal(gl);
+    if (obs) {
+        rows_free(rm);
+        if (m.act) {
+            float2* o2 = reinterpret_cast<float2*>(rows + rm.off + row_shift(rm, obs, od) + rm.rank * od);
+            o2[0] = make_float2(s.x[0] - gl[0] + ex[0], s.x[1] - gl[1] + ex[1]);
+            o2[1] = make_float2(s.x[2] - gl[2] + ex[2], s.v[0] + evv[0]);
+            o2[2] = make_float2(s.v[1] + evv[1], s.v[2] + evv[2]);
+            o2[3] = make_float2(s.R[0], s.R[1]);
+            o2[4] = make_float2(s.R[2], s.R[3]);
+            o2[5] = make_float2(s.R[4], s.R[5]);
+            o2[6] = make_float2(s.R[6], s.R[7]);
+            o2[7] = make_float2(s.R[8], s.w[0] + ew[0]);
+            o2[8] = make_float2(s.w[1] + ew[1], s.w[2] + ew[2]);
+#pragma unroll
+            for (int k = 0; k < QS_MAX_K; ++k) {
+                if (k >= K) break;
+                float2* on = o2 + 9 + 3 * k;
+                if (k < keff) {
+                    const int j = nbr_at(nb, k);
+                    const float4 q = sh.px[b][j];
+                    const float2 v = sh.vyz[b][j];
+                    on[0] = make_float2(q.x - s.x[0], q.y - s.x[1]);
+                    on[1] = make_float2(q.z - s.x[2], q.w - s.v[0]);
+                    on[2] = make_float2(v.x - s.v[1], v.y - s.v[2]);
+                } else {
+                    on[0] = make_float2(0.f, 0.f);
+                    on[1] = make_float2(0.f, 0.f);
+                    on[2] = make_float2(0.f, 0.f);
+                }
+            }
+        }
+        send_rows(rm, rows, obs, od, bulk);
     }
-    const float g[3] = {sh.g[b][0][L], sh.g[b][1][L], sh.g[b][2][L]};
-    const NbrList nb = sh.nb[b][L];
-    rew[m.d] = compute_reward(c, s, sh.rin[b][8][L], g, fh, sh.ev[b][L], sh.keff[b][L], [&](int k) {
-        const int j = nbr_at(nb, k);
-        return make_float3(sh.st[b][0][j], sh.st[b][1][j], sh.st[b][2][j]);
-    });
+    if (rew && m.act) {
+        const float4 f = sh.fh[b][L], p = sh.fp[b][L];
+        const float2 pe = sh.pe[b][L];
+        const float fh[4] = {f.x, f.y, f.z, f.w};
+        s.fp[0] = p.x; s.fp[1] = p.y; s.fp[2] = p.z; s.fp[3] = p.w;
+        rew[m.d] = compute_reward(c, s, pe.x, gl, fh, __float_as_uint(pe.y), keff, [&](int k) {
+            const float4 q = sh.px[b][nbr_at(nb, k)];
+            return make_float3(q.x, q.y, q.z);
+        });
+    }
+}
+
+// The noise warp's rows in dynamic shared memory.
+__device__ __forceinline__ float* ws_rows(const Consts& c, int L) {
+    extern __shared__ float4 sm[];
+    return reinterpret_cast<float*>(sm) + (L & ~31) * (c.obs_dim + ROW_PAD);
 }
 
 template <bool EXT>
@@ -888,7 +869,9 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
         if (m.act && io.obs && (c.flags & QS_F_OBS_NOISE)) obs_noise(c, tick, m.d, 0u, ex, evv, ew);
         __syncthreads();  // B2
         launch_next();
-        if (io.obs) ws_store_obs<1>(c, dv, tile, perm, sh, m, 0, io.obs, ex, evv, ew);
+        if (io.obs)
+            ws_finish<1>(c, sh, m, map_rows(m.act, m.d, m.W, c.obs_dim), ws_rows(c, m.L), 0, io.obs, nullptr, false, ex, evv, ew,
+                         [](float*) {});
         return;
     }
     // ---------------- dynamics warp
@@ -943,22 +926,20 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
         const bool scn = EXT && (c.scn_mask & ~1u) != 0;
         int ep = scn && m.act ? dv.ep[m.e] : 0, sel = scn && m.act ? dv.scn_sel[m.e] : 0;
         GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
-        // finishes the step published in buffer b (time t0 + t): goals, rows, rewards
+        const RowMap rm = map_rows(m.act, m.d, m.W, c.obs_dim);
+        float* rows = ws_rows(c, m.L);
         const auto finish = [&](int t) {
-            const int b = t & 1;
-            if (scn) {
-                float gl[3] = {sh.g[b][0][m.L], sh.g[b][1][m.L], sh.g[b][2][m.L]};
+            ws_finish<P>(c, sh, m, rm, rows, t & 1, io.obs ? io.obs + (size_t)(t0 + t) * D * c.obs_dim : nullptr,
+                         io.rew ? io.rew + (size_t)(t0 + t) * D : nullptr, io.bulk, px, pv, pw, [&](float* gl) {
+                if (!scn) return;
                 ws_goal<P>(c, dv, sh, m, sel, ep + 1, gc, gl, 2);
-                for (int k = 0; k < 3; ++k) sh.g[b][k][m.L] = gl[k];
                 ep = ep + 1;
                 if (ep >= c.episode_steps && (c.flags & QS_F_AUTO_RESET)) {
                     ep = 0;
                     sel ^= 1;
                     gc.until = -1;
                 }
-            }
-            if (io.obs) ws_store_obs<P>(c, dv, tile, perm, sh, m, b, io.obs + (size_t)(t0 + t) * D * c.obs_dim, px, pv, pw);
-            if (io.rew) ws_reward<P>(c, sh, m, b, io.rew + (size_t)(t0 + t) * D);
+            });
         };
         for (int t = 0; t < nsteps; ++t) {
             // buffer t & 1 holds step t's normals, drawn before B2 of step t - 1:
@@ -981,6 +962,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const C
         }
         launch_next();
         if (nsteps > 0) finish(nsteps - 1);  // after the last B2
+        if (rm.lead) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
         return;
     }
     // ---------------- dynamics side
@@ -1125,6 +1107,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_serve(const Consts
         load_drone(s, dv.st, dv.D, m.d);
         load_env<EXT>(er, c, dv, m.e);
     }
+    const RowMap rm = map_rows(m.act, m.d, m.W, c.obs_dim);
     if (noise) ws_motor_normals<P>(c, sh, m, tick0, 0);
     for (int k = 0;; ++k) {
         if (threadIdx.x == 0) {
@@ -1146,7 +1129,7 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_serve(const Consts
             float ex[3] = {0.f, 0.f, 0.f}, evv[3] = {0.f, 0.f, 0.f}, ew[3] = {0.f, 0.f, 0.f};
             if (m.act && io.obs && (c.flags & QS_F_OBS_NOISE)) obs_noise(c, tick, m.d, 0u, ex, evv, ew);
             __syncthreads();  // B2
-            if (io.obs) ws_store_obs<P>(c, dv, tile, perm, sh, m, b, io.obs, ex, evv, ew);
+            if (io.obs) ws_finish<P>(c, sh, m, rm, ws_rows(c, m.L), b, io.obs, nullptr, false, ex, evv, ew, [](float*) {});
             ws_motor_normals<P>(c, sh, m, tick + 1, b ^ 1);
         } else {
             // the host's commands of this step: fetched again, never from a cached line
@@ -1183,7 +1166,7 @@ cudaError_t launch_serve(const Consts& c, const Dev& dv, const Tile* tiles, int 
     const int* pp = perm;
     int kk = k0;
     void* args[] = {&cc, &dd, &tt, &pp, &ii, &kk};
-    return cudaLaunchCooperativeKernel(fn, dim3(n_tiles), dim3(64 * P), args, 0, st);
+    return cudaLaunchCooperativeKernel(fn, dim3(n_tiles), dim3(64 * P), args, ws_smem(c, P), st);
 }
 
 int serve_resident_ctas(const Consts& c, int P) {
@@ -1193,7 +1176,7 @@ int serve_resident_ctas(const Consts& c, int P) {
     const bool ext = extended(c);
     const void* fn = P == 1 ? (ext ? (const void*)k_serve<true, 1> : (const void*)k_serve<false, 1>)
                             : (ext ? (const void*)k_serve<true, 2> : (const void*)k_serve<false, 2>);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess) return 0;
     return occ * n_sm;
 }
 
@@ -1204,7 +1187,7 @@ int rollout_ws_resident_ctas(const Consts& c, int P) {
     const bool ext = extended(c);
     const void* fn = P == 1 ? (ext ? (const void*)k_rollout_ws<true, 1> : (const void*)k_rollout_ws<false, 1>)
                             : (ext ? (const void*)k_rollout_ws<true, 2> : (const void*)k_rollout_ws<false, 2>);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, 0) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess) return 0;
     return occ * n_sm;
 }
 
@@ -1244,7 +1227,8 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
     if (cp.n_tiles == 0) return cudaSuccess;
     const bool ext = extended(c);
     if (cp.ws && !observe_only)
-        return launch_overlapped(ext ? k_step_ws<true> : k_step_ws<false>, cp.n_tiles, 64, 0, st, c, dv, tiles + cp.tile_off,
+        return launch_overlapped(ext ? k_step_ws<true> : k_step_ws<false>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
+                                 tiles + cp.tile_off,
                                  perm, io);
     const size_t smem = (cp.W > 1) ? sizeof(float) * SMEM_PLANES * cp.block : 0;
     const Tile* t = tiles + cp.tile_off;
@@ -1291,7 +1275,7 @@ cudaError_t launch_rollout_ws(const Consts& c, const Dev& dv, const Tile* tiles,
     if (P != 1 && P != 2) return cudaErrorInvalidValue;
     const auto k = P == 1 ? (ext ? k_rollout_ws<true, 1> : k_rollout_ws<false, 1>)
                           : (ext ? k_rollout_ws<true, 2> : k_rollout_ws<false, 2>);
-    return launch_overlapped(k, n_tiles, 64 * P, 0, st, c, dv, tiles, perm, io, t0, nsteps);
+    return launch_overlapped(k, n_tiles, 64 * P, ws_smem(c, P), st, c, dv, tiles, perm, io, t0, nsteps);
 }
 
 cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int block, const int* perm,
