@@ -353,7 +353,8 @@ bool device_memory(const void* p) {
 // -> 35.5 us, 65,536 envs 271 -> 207 us); one class keeps its per-call kernel.
 qs_status do_step(qs_env* h, const float* act, float* obs, float* rew, uint8_t* done) {
     if (h->plan.size() > 1) return enqueue_rollout(h, 1, RolloutIO{act, obs, rew, done, false});
-    StepIO io{act, obs, rew, done};
+    // (only the one-thread-per-drone step of single drones sends bulk copies)
+    StepIO io{act, obs, rew, done, h->single_drone && !h->plan[0].ws && device_memory(obs)};
     for (const ClassPlan& cp : h->plan) {
         cudaError_t e = launch_step(h->c, h->dv, cp, h->d_tiles, h->d_perm, io, 0, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
@@ -551,7 +552,7 @@ qs_status qs_create(const qs_config* cfg, void* cuda_stream, qs_env** out) {
         off = o + bytes;
         return o;
     };
-    const size_t o_st = take(sizeof(float4) * NPLANE * D), o_prm = take(sizeof(float) * NPRM_DEV * E),
+    const size_t o_st = take((sizeof(float4) * NPLANE_PUBLIC + sizeof(float)) * D), o_prm = take(sizeof(float) * NPRM_DEV * E),
                  o_goal = take(sizeof(float) * 3 * E), o_ep = take(sizeof(int32_t) * E),
                  o_tick = take(sizeof(uint32_t) * E), o_off = take(sizeof(int32_t) * (E + 1)),
                  o_of = take(sizeof(int32_t) * D), o_ev = take(sizeof(uint32_t) * D),
@@ -670,7 +671,7 @@ qs_status qs_reset(qs_env* h, uint64_t seed, const uint8_t* env_mask_dev, float*
     cudaError_t e = launch_reset(h->c, h->dv, k0, k1, env_mask_dev, h->stream);
     if (e != cudaSuccess) return cuda_fail(h, e, "qs_reset launch");
     if (obs_dev) {
-        StepIO io{nullptr, obs_dev, nullptr, nullptr};
+        StepIO io{nullptr, obs_dev, nullptr, nullptr, false};
         for (const ClassPlan& cp : h->plan) {
             e = launch_step(h->c, h->dv, cp, h->d_tiles, h->d_perm, io, 1, h->stream);
             if (e != cudaSuccess) return cuda_fail(h, e, "qs_reset observation");

@@ -381,18 +381,29 @@ __device__ __forceinline__ void comp_add_prod(float& hi, float& lo, float a, flo
     hi = t;
 }
 
-__device__ __forceinline__ void load_drone(Drone& s, const float4* __restrict__ st, int D, int d) {
+// A drone's state in memory: planes of float4 [D] that hold the 30 public floats
+// and, in the two that remain of the last, the low-order parts of w_x and w_y,
+// then a plane of float [D] with that of w_z: 132 bytes a drone (144 with a
+// ninth float4 plane for the low-order parts; a step of 1,048,576 single
+// drones, which memory bounds, 84.0 -> 83.3 us).
+__device__ __forceinline__ float* low_plane(float4* st, int D) { return reinterpret_cast<float*>(st + (size_t)NPLANE_PUBLIC * D); }
+
+__device__ __forceinline__ void load_drone(Drone& s, float4* st, int D, int d) {
     float4 q[NPLANE];
 #pragma unroll
-    for (int p = 0; p < NPLANE; ++p) q[p] = st[(size_t)p * D + d];
+    for (int p = 0; p < NPLANE_PUBLIC; ++p) q[p] = st[(size_t)p * D + d];
+    q[NPLANE_PUBLIC] = make_float4(q[NPLANE_PUBLIC - 1].z, q[NPLANE_PUBLIC - 1].w, low_plane(st, D)[d], 0.f);
     unpack(s, q);
 }
 
-__device__ __forceinline__ void store_drone(const Drone& s, float4* __restrict__ st, int D, int d) {
+__device__ __forceinline__ void store_drone(const Drone& s, float4* st, int D, int d) {
     float4 q[NPLANE];
     pack(s, q);
+    q[NPLANE_PUBLIC - 1].z = s.wlo[0];
+    q[NPLANE_PUBLIC - 1].w = s.wlo[1];
 #pragma unroll
-    for (int p = 0; p < NPLANE; ++p) st[(size_t)p * D + d] = q[p];
+    for (int p = 0; p < NPLANE_PUBLIC; ++p) st[(size_t)p * D + d] = q[p];
+    low_plane(st, D)[d] = s.wlo[2];
 }
 
 // Initial drone state (Sec. III-A with DR): position uniform in the room,

@@ -23,9 +23,10 @@ enum Tag : uint32_t {
     TAG_SWAP = 13
 };
 
-// Number of float4 planes of the drone state: the 30 public floats fill
-// planes 0..7 (2 pad); plane 8 holds the low-order parts of the body rates
-// (compensated accumulation, see Drone::wlo) and 1 pad.
+// Number of float4 planes of a drone's packed state (the differentiable
+// rollout's checkpoints): the 30 public floats fill planes 0..7 (2 pad); plane
+// 8 holds the low-order parts of the body rates (compensated accumulation, see
+// Drone::wlo) and 1 pad. A handle's own state is packed closer (load_drone).
 constexpr int NPLANE = 9;
 constexpr int NPLANE_PUBLIC = 8;
 
@@ -71,7 +72,7 @@ inline void set_round_keys(Consts& c) {
 
 // Device buffers owned by a handle.
 struct Dev {
-    float4* st;              // [NPLANE][D] drone state planes
+    float4* st;              // drone state: float4 [NPLANE_PUBLIC][D], float [D] (load_drone)
     float* prm;              // [NPRM_DEV][E]
     float* goal;             // [3][E]
     int32_t* ep;             // [E] control steps into the episode
@@ -114,6 +115,7 @@ struct StepIO {
     float* obs;        // [D][obs_dim] or null
     float* rew;        // [D] or null
     uint8_t* done;     // [E] or null
+    bool bulk;         // obs is device memory (rows may leave by bulk asynchronous copies)
 };
 
 // [T][...] buffers of a rollout (outputs nullable).

@@ -53,8 +53,8 @@ cudaError_t launch_reset(const Consts& c, const Dev& dv, uint32_t k0, uint32_t k
 __global__ void k_get_drones(const Dev dv, float* __restrict__ out) {
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= dv.D) return;
-    float4 q[NPLANE];
-    for (int p = 0; p < NPLANE; ++p) q[p] = dv.st[(size_t)p * dv.D + d];
+    float4 q[NPLANE_PUBLIC];
+    for (int p = 0; p < NPLANE_PUBLIC; ++p) q[p] = dv.st[(size_t)p * dv.D + d];
     const float* f = reinterpret_cast<const float*>(q);
     for (int k = 0; k < QS_STATE_DIM; ++k) out[(size_t)d * QS_STATE_DIM + k] = f[k];
 }
@@ -80,11 +80,12 @@ cudaError_t launch_get_state(const Dev& dv, float* state, float* params, float* 
 __global__ void k_set_drones(const Dev dv, const float* __restrict__ in) {
     const int d = blockIdx.x * blockDim.x + threadIdx.x;
     if (d >= dv.D) return;
-    float4 q[NPLANE];
+    float4 q[NPLANE_PUBLIC];
     float* f = reinterpret_cast<float*>(q);
     for (int k = 0; k < QS_STATE_DIM; ++k) f[k] = in[(size_t)d * QS_STATE_DIM + k];
-    for (int k = QS_STATE_DIM; k < 4 * NPLANE; ++k) f[k] = 0.f;  // pads and body-rate low parts
-    for (int p = 0; p < NPLANE; ++p) dv.st[(size_t)p * dv.D + d] = q[p];
+    for (int k = QS_STATE_DIM; k < 4 * NPLANE_PUBLIC; ++k) f[k] = 0.f;  // body-rate low parts
+    for (int p = 0; p < NPLANE_PUBLIC; ++p) dv.st[(size_t)p * dv.D + d] = q[p];
+    low_plane(dv.st, dv.D)[d] = 0.f;
 }
 
 __global__ void k_set_envs(const Consts c, const Dev dv, const float* params, const float* goals, const int32_t* ep,

@@ -461,12 +461,19 @@ __global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(con
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
     float gv[GOAL_VALUES];
     GoalCache gc{gv, GOAL_FIXED, 0, -1};
-    step_body<EXT, false>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
-              io.rew, io.done, observe_only, gc, RowMap(), nullptr, false);
-    if (!m.act || observe_only) return;
-    dv.ev[m.d] = ev;
-    store_drone(s, dv.st, dv.D, m.d);
-    if (m.lane == 0) store_env<EXT>(er, dv, m.e);
+    // single drones: rows of a warp as one block (see RowMap; 65,536 drones 8.0 ->
+    // 7.7 us, 1,048,576 83.3 -> 82.5 us)
+    constexpr bool ROWS = W == 1 && !EXT;
+    const RowMap rm = ROWS ? map_rows(m.act, m.d, 1, c.obs_dim) : RowMap();
+    float* rows = reinterpret_cast<float*>(sm) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
+    step_body<EXT, ROWS>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
+              io.rew, io.done, observe_only, gc, rm, rows, io.bulk);
+    if (m.act && !observe_only) {
+        dv.ev[m.d] = ev;
+        store_drone(s, dv.st, dv.D, m.d);
+        if (m.lane == 0) store_env<EXT>(er, dv, m.e);
+    }
+    if (ROWS && rm.lead) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
 // T steps of one tile with the state in registers. W1: every tile of the
@@ -1191,6 +1198,13 @@ int rollout_ws_resident_ctas(const Consts& c, int P) {
     return occ * n_sm;
 }
 
+// A kernel whose shared memory passes the 48 KiB every kernel may have (large
+// CTAs with many neighbours) asks for the most any shape needs, so that no
+// handle's call lowers another's.
+cudaError_t allow_smem(const void* fn, size_t smem) {
+    return smem <= 48u << 10 ? cudaSuccess : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM_MAX);
+}
+
 // CTAs of `block` threads of the single-drone step (80 registers) in a wave.
 int step_wave(int block) {
     int dev = 0, n_sm = 152;
@@ -1207,6 +1221,9 @@ cudaError_t launch_k_step(const Consts& c, const Dev& dv, const ClassPlan& cp, c
     };
     switch (cp.W) {
         case 1: {
+            cudaError_t e = allow_smem((const void*)k_step<1, EXT>, smem);
+            if (e == cudaSuccess) e = allow_smem((const void*)k_step<1, EXT, false>, smem);
+            if (e != cudaSuccess) return e;
             if (cp.n_tiles <= STEP_OVERLAP_WAVES * step_wave(cp.block)) return k(k_step<1, EXT>);
             k_step<1, EXT, false><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only);
             return cudaGetLastError();
@@ -1230,7 +1247,9 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
         return launch_overlapped(ext ? k_step_ws<true> : k_step_ws<false>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
                                  tiles + cp.tile_off,
                                  perm, io);
-    const size_t smem = (cp.W > 1) ? sizeof(float) * SMEM_PLANES * cp.block : 0;
+    const size_t smem = cp.W > 1 ? sizeof(float) * SMEM_PLANES * cp.block
+                        : ext     ? 0
+                                  : sizeof(float) * cp.block * (c.obs_dim + ROW_PAD);
     const Tile* t = tiles + cp.tile_off;
     return ext ? launch_k_step<true>(c, dv, cp, t, perm, io, observe_only, smem, st)
                : launch_k_step<false>(c, dv, cp, t, perm, io, observe_only, smem, st);
@@ -1241,13 +1260,6 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
 const void* rollout_kernel(bool ext, bool single) {
     if (ext) return (const void*)k_rollout<true, false>;
     return single ? (const void*)k_rollout<false, true> : (const void*)k_rollout<false, false>;
-}
-
-// A rollout kernel whose shared memory passes the 48 KiB every kernel may have (large
-// CTAs with many neighbours) asks for the most any shape needs, so that no
-// handle's call lowers another's.
-cudaError_t allow_smem(const void* fn, size_t smem) {
-    return smem <= 48u << 10 ? cudaSuccess : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM_MAX);
 }
 
 // Its dynamic shared memory: two sets of staging planes and the CTA's
