@@ -52,11 +52,12 @@ struct Consts {
     int substeps, K, episode_steps, obs_dim;
 };
 
-// Whether a handle runs the general instance of the step kernels (scenario
-// goals, downwash or smooth contacts, each decided at run time) rather than
-// the common one that compiles them out.
-inline bool extended_instance(const Consts& c) {
-    return (c.scn_mask & ~1u) != 0 || (c.flags & (QS_F_DOWNWASH | QS_F_SMOOTH)) != 0;
+// The instance of the step kernels a handle runs: 0 the common one, 1 with
+// scenario goals and downwash (each decided at run time), 2 that with the smooth
+// contacts.
+inline int extended_instance(const Consts& c) {
+    if (c.flags & QS_F_SMOOTH) return 2;
+    return (c.scn_mask & ~1u) != 0 || (c.flags & QS_F_DOWNWASH) != 0 ? 1 : 0;
 }
 
 // Fills c.rk from c.key0 / c.key1 (Weyl increments 0x9E3779B9, 0xBB67AE85).

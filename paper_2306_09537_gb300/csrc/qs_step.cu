@@ -36,13 +36,15 @@ constexpr int ROW_PAD = 6;
 // and the most the kernels ask for
 constexpr int STEP_SMEM_MAX = (int)sizeof(float) * MAX_BLOCK * (2 * SMEM_PLANES + GOAL_STRIDE + 18 + 6 * QS_MAX_K + ROW_PAD);
 
-// The step kernels come in two instances: EXT = true carries the training
-// scenarios (per-drone goals), the downwash term and the smooth contacts,
-// deciding each at run time; EXT = false is the common configuration (one
-// goal, no downwash, the paper's discrete contacts) with these decided at
-// compile time, so it keeps the smaller code and register budget, and the
-// substep's contact branch is straight-line code (extended_instance()).
-inline bool extended(const Consts& c) { return extended_instance(c); }
+// The step kernels come in three instances, EXT = extended_instance(): 0 the
+// common configuration (one goal, no downwash, the paper's discrete contacts)
+// with all of it decided at compile time, so it keeps the smaller code and
+// register budget and the substep's contact branch is straight-line code; 1
+// with the training scenarios (per-drone goals) and the downwash term, decided
+// at run time; 2 that with the smooth contacts in place of the discrete ones.
+// (Deciding the contacts at run time too, the dynamics side of 1999 swarms of 7
+// under every scenario took 4,600 cycles for its substeps against 3,700.)
+inline int extended(const Consts& c) { return extended_instance(c); }
 
 // Per-env values a thread keeps in registers.
 struct EnvRegs {
@@ -54,7 +56,7 @@ struct EnvRegs {
     bool redrawn;  // auto-reset drew new parameters / goal this launch
 };
 
-template <bool EXT>
+template <int EXT>
 __device__ __forceinline__ void load_env(EnvRegs& er, const Consts& c, const Dev& dv, int e) {
     er.p = load_prm(c, dv.prm, dv.E, e);
     er.g0 = dv.goal[e];
@@ -67,7 +69,7 @@ __device__ __forceinline__ void load_env(EnvRegs& er, const Consts& c, const Dev
 }
 
 // Written by lane 0 of the slot at the end of a launch.
-template <bool EXT>
+template <int EXT>
 __device__ __forceinline__ void store_env(const EnvRegs& er, const Dev& dv, int e) {
     dv.ep[e] = er.ep;
     dv.tick[e] = er.tick;
@@ -153,7 +155,7 @@ __device__ __forceinline__ float compute_reward(const Consts& c, const Drone& s,
 
 // End of a control step: previous command, episode counter, done flag,
 // Philox counter, in-place auto-reset, non-finite check.
-template <bool EXT>
+template <int EXT>
 __device__ __forceinline__ void end_step(const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, const float fh[4],
                                          int lane, int e, int d, uint8_t* __restrict__ done) {
     s.fp[0] = fh[0];
@@ -269,7 +271,7 @@ __device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, fl
 // steps, 358 -> 299 us; 256 x 128, 16 steps, 203 -> 183 us); single drones keep
 // their 9 stores: addressing the block costs 95 instructions of 1,100 a step,
 // more than the stores' waits (1,048,576 drones, 32 steps: 1696 against 1834 us).
-template <bool EXT, bool ROWS>
+template <int EXT, bool ROWS>
 __device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, uint32_t& ev_out,
                                           float4* sp, float* sv, const bool act, const int lane, const int N,
                                           const int sbase, const int e, const int d, const float4 a,
@@ -279,7 +281,7 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
     const int K = c.K;
     const int keff = min(K, N - 1);
     const uint32_t tick = er.tick;
-    // the EXT = false instance carries neither scenario nor downwash code
+    // the EXT = 0 instance carries neither scenario nor downwash code
     const bool scn = EXT && (c.scn_mask & ~1u) != 0;
     const bool dw = EXT && (c.flags & QS_F_DOWNWASH) != 0;
     const int tau = observe_only ? er.ep : er.ep + 1;  // the goal is the one at the step's end
@@ -291,7 +293,7 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
     // smooth contacts of a swarm (general instance): the pair penalty from the
     // positions at each substep's start, staged like the pair pass (uniform
     // over the CTA: every thread meets the barriers)
-    const bool spair = EXT && (c.flags & QS_F_SMOOTH) && W > 1 && !observe_only;
+    const bool spair = EXT == 2 && W > 1 && !observe_only;
     if (spair) {
         if (act) {
             fh[0] = command(c, a.x);
@@ -306,7 +308,7 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
             __syncthreads();
             if (act && N > 1) pair_acc(c, s.x, sp, sbase, lane, N, er.p.arm, pacc);
             __syncthreads();
-            if (act) ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, tick, d, sub, pacc);
+            if (act) ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, tick, d, sub, pacc);
         }
     } else if (act && !observe_only) {
         fh[0] = command(c, a.x);
@@ -315,7 +317,7 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         fh[3] = command(c, a.w);
         const float u[4] = {sqrt_approx(fh[0]), sqrt_approx(fh[1]), sqrt_approx(fh[2]), sqrt_approx(fh[3])};
         const float zero3[3] = {0.f, 0.f, 0.f};
-        for (int sub = 0; sub < c.substeps; ++sub) ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, tick, d, sub, zero3);
+        for (int sub = 0; sub < c.substeps; ++sub) ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, tick, d, sub, zero3);
     }
 
     // ---- pair pass: collisions (S9, S10) and K nearest neighbours (S11)
@@ -332,9 +334,9 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         bool responded = false, dw_hit = false;
         float dw_az = 0.f;
         if (act && N > 1) {
-            const bool coll = (c.flags & QS_F_COLLISIONS) && !(EXT && (c.flags & QS_F_SMOOTH)) && !observe_only;
+            const bool coll = (c.flags & QS_F_COLLISIONS) && EXT != 2 && !observe_only;
             const bool flag_coll = (c.flags & QS_F_COLLISIONS) && !observe_only;
-            responded = pair_scan<EXT>(c, s, er.p.thr, lane, N, sbase, sp, sv, nt, keff, coll, flag_coll, ev, nbrs, dvs,
+            responded = pair_scan<(EXT > 0)>(c, s, er.p.thr, lane, N, sbase, sp, sv, nt, keff, coll, flag_coll, ev, nbrs, dvs,
                                        dw && !observe_only, dw_az, dw_hit);
         }
         if (responded) apply_response(c, s, tick, d, dvs);
@@ -444,7 +446,7 @@ __device__ __forceinline__ SlotMap map_slot(const Dev& dv, const Tile& tile, con
 // drones 10.3 -> 8.0 us a step, 262,144 28.7 -> 28.3); past them every CTA's
 // wait costs more than the launch (1,048,576: 83.2 -> 87.9 us).
 constexpr int STEP_OVERLAP_WAVES = 2;
-template <int W, bool EXT, bool OVERLAP = true>
+template <int W, int EXT, bool OVERLAP = true>
 __global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                     const int* __restrict__ perm, const StepIO io, const int observe_only) {
     extern __shared__ float4 sm[];
@@ -479,7 +481,7 @@ __global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(con
 // T steps of one tile with the state in registers. W1: every tile of the
 // launch holds single-drone slots (a compile-time width of 1: no pair pass,
 // neighbour or staging code).
-template <bool EXT, bool W1>
+template <int EXT, bool W1>
 __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, const Tile& tile, const int* __restrict__ perm,
                                              float4* sm, const RolloutIO& io, int t0, int nsteps) {
     const int W = W1 ? 1 : tile.W;
@@ -520,15 +522,15 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
 // CTA draws one number past the tiles, and the last of those puts the counter
 // back to zero for the next launch (a memset before each launch cost a launch
 // of its own). Tiles are ordered costliest first. The W1 instance
-// (EXT = false only) serves handles whose envs all hold one drone: 107
+// (EXT = 0 only) serves handles whose envs all hold one drone: 107
 // registers instead of 121 and no untaken swarm code in the step loop (with
-// the smooth contacts compiled out of the EXT = false instances, batched
+// the smooth contacts compiled out of the EXT = 0 instances, batched
 // 1,048,576 single-drone envs went from 1.75e10 to 1.90e10 quadrotor-steps/s,
 // each change about half of it). Held to 104 registers it fits in 96 without a
 // spill, five warps a scheduler instead of four (1,048,576 drones, 32 steps,
 // 1687 -> 1632 us, in 32-thread CTAs 1593; at 88 registers 1644). Swarms spill
 // below 128 (16,384 x 8, 64 steps: 128 registers 746 us, 112 799, 160 901).
-template <bool EXT, bool W1>
+template <int EXT, bool W1>
 __global__ void __maxnreg__(W1 ? 104 : 128) k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                        const int n_tiles, const int* __restrict__ perm,
                                                        int* __restrict__ counter, const RolloutIO io, const int t0,
@@ -667,7 +669,7 @@ __device__ __forceinline__ void ws_goal(const Consts& c, const Dev& dv, WsShared
 // and B2 (post-step state, goal and neighbours published for the observation
 // rows), then writes the knn record, reward and done and ends the step. Every
 // thread of the dynamics warps calls it.
-template <bool EXT, int P, bool DEFER>
+template <int EXT, int P, bool DEFER>
 __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv, WsShared<P>& sh, const WsMap& m,
                                                  Drone& s, EnvRegs& er, uint32_t& ev_out, const float4 a, const int nb,
                                                  float* __restrict__ rew, uint8_t* __restrict__ done, GoalCache& gc,
@@ -678,7 +680,7 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
     const int K = c.K;
     const int nahead = min(c.substeps, WS_SUB);
     const bool mnoise = (c.flags & QS_F_MOTOR_NOISE) != 0;
-    const bool dw = EXT && (c.flags & QS_F_DOWNWASH) != 0;  // EXT = false: no downwash or scenario code
+    const bool dw = EXT && (c.flags & QS_F_DOWNWASH) != 0;  // EXT = 0: no downwash or scenario code
     float fh[4] = {0.f, 0.f, 0.f, 0.f}, u[4] = {0.f, 0.f, 0.f, 0.f};
     uint32_t ev = 0;
     if (act) {
@@ -694,7 +696,7 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
     if (b1) __syncthreads();  // B1: motor normals ready (the rollout's later steps: drawn before the last B2)
     // smooth contacts of a swarm (general instance): the pair penalty from the
     // positions at each substep's start, staged like the pair pass
-    const bool spair = EXT && (c.flags & QS_F_SMOOTH) && W > 1;
+    const bool spair = EXT == 2 && W > 1;
     if (spair) {
         for (int sub = 0; sub < c.substeps; ++sub) {
             float pacc[3] = {0.f, 0.f, 0.f};
@@ -706,9 +708,9 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
                 if (mnoise && sub < nahead) {
                     const float4 q = sh.nrm[nb][sub][L];
                     const float n[4] = {q.x, q.y, q.z, q.w};
-                    ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, pacc, n);
+                    ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, er.tick, d, sub, pacc, n);
                 } else {
-                    ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, pacc);
+                    ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, er.tick, d, sub, pacc);
                 }
             }
         }
@@ -718,9 +720,9 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
             if (mnoise && sub < nahead) {
                 const float4 q = sh.nrm[nb][sub][L];
                 const float n[4] = {q.x, q.y, q.z, q.w};
-                ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, zero3, n);
+                ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, er.tick, d, sub, zero3, n);
             } else {
-                ev |= substep<false, EXT ? -1 : 0>(s, er.p, c, u, er.tick, d, sub, zero3);
+                ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, er.tick, d, sub, zero3);
             }
         }
     }
@@ -738,9 +740,9 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         bool responded = false, dw_hit = false;
         float dw_az = 0.f;
         if (act && N > 1) {
-            const bool coll = (c.flags & QS_F_COLLISIONS) && !(EXT && (c.flags & QS_F_SMOOTH));
+            const bool coll = (c.flags & QS_F_COLLISIONS) && EXT != 2;
             const bool flag_coll = (c.flags & QS_F_COLLISIONS) != 0;
-            responded = pair_scan<EXT>(c, s, er.p.thr, lane, N, sbase, sh.sp, &sh.sv[0][0], 32 * P, keff, coll, flag_coll,
+            responded = pair_scan<(EXT > 0)>(c, s, er.p.thr, lane, N, sbase, sh.sp, &sh.sv[0][0], 32 * P, keff, coll, flag_coll,
                                        ev, nbrs, dvs, dw, dw_az, dw_hit);
         }
         if (responded) apply_response(c, s, er.tick, d, dvs);
@@ -860,7 +862,7 @@ __device__ __forceinline__ float* ws_rows(const Consts& c, int L) {
     return reinterpret_cast<float*>(sm) + (L & ~31) * (c.obs_dim + ROW_PAD);
 }
 
-template <bool EXT>
+template <int EXT>
 __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                 const int* __restrict__ perm, const StepIO io) {
     __shared__ WsShared<1> sh;
@@ -910,7 +912,7 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
 // a step overlaps the dynamics side's end of the previous one (plain 8192 /
 // 4864 / 2432 envs: +2% / +5% / +7%); swarm slots meet at B1 and B2 of every
 // step (without B1, 3.56e9 -> 3.50e9 quadrotor-steps/s for 2048 x 8).
-template <bool EXT, int P>
+template <int EXT, int P>
 __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                        const int* __restrict__ perm, const RolloutIO io, const int t0,
                                                        const int nsteps) {
@@ -1097,7 +1099,7 @@ __device__ __forceinline__ unsigned long long serve_wait(unsigned long long* go,
 // by the noise side after B2 and the next step's normals drawn after them,
 // then B3, after which thread 0 fences the CTA's host writes at system scope
 // and counts the CTA done; the last CTA publishes fin = k0 + k + 1.
-template <bool EXT, int P>
+template <int EXT, int P>
 __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_serve(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                                   const int* __restrict__ perm, const ServeIO io, const int k0) {
     __shared__ WsShared<P> sh;
@@ -1160,11 +1162,20 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_serve(const Consts
     if (m.lane == 0) store_env<EXT>(er, dv, m.e);
 }
 
+// The instance of a warp-specialised kernel for a handle (ext: extended()).
+template <int P>
+const void* serve_kernel(int ext) {
+    return ext == 2 ? (const void*)k_serve<2, P> : ext == 1 ? (const void*)k_serve<1, P> : (const void*)k_serve<0, P>;
+}
+template <int P>
+auto rollout_ws_kernel(int ext) {
+    return ext == 2 ? k_rollout_ws<2, P> : ext == 1 ? k_rollout_ws<1, P> : k_rollout_ws<0, P>;
+}
+
 cudaError_t launch_serve(const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int P, const int* perm,
                          const ServeIO& io, int k0, cudaStream_t st) {
-    const bool ext = extended(c);
-    const void* fn = P == 1 ? (ext ? (const void*)k_serve<true, 1> : (const void*)k_serve<false, 1>)
-                            : (ext ? (const void*)k_serve<true, 2> : (const void*)k_serve<false, 2>);
+    const int ext = extended(c);
+    const void* fn = P == 1 ? serve_kernel<1>(ext) : serve_kernel<2>(ext);
     if (P != 1 && P != 2) return cudaErrorInvalidValue;
     Consts cc = c;
     Dev dd = dv;
@@ -1180,9 +1191,8 @@ int serve_resident_ctas(const Consts& c, int P) {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const bool ext = extended(c);
-    const void* fn = P == 1 ? (ext ? (const void*)k_serve<true, 1> : (const void*)k_serve<false, 1>)
-                            : (ext ? (const void*)k_serve<true, 2> : (const void*)k_serve<false, 2>);
+    const int ext = extended(c);
+    const void* fn = P == 1 ? serve_kernel<1>(ext) : serve_kernel<2>(ext);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess) return 0;
     return occ * n_sm;
 }
@@ -1191,9 +1201,8 @@ int rollout_ws_resident_ctas(const Consts& c, int P) {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const bool ext = extended(c);
-    const void* fn = P == 1 ? (ext ? (const void*)k_rollout_ws<true, 1> : (const void*)k_rollout_ws<false, 1>)
-                            : (ext ? (const void*)k_rollout_ws<true, 2> : (const void*)k_rollout_ws<false, 2>);
+    const int ext = extended(c);
+    const void* fn = P == 1 ? (const void*)rollout_ws_kernel<1>(ext) : (const void*)rollout_ws_kernel<2>(ext);
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess) return 0;
     return occ * n_sm;
 }
@@ -1213,7 +1222,7 @@ int step_wave(int block) {
     return n_sm * (768 / block);
 }
 
-template <bool EXT>
+template <int EXT>
 cudaError_t launch_k_step(const Consts& c, const Dev& dv, const ClassPlan& cp, const Tile* t, const int* perm,
                           const StepIO& io, int observe_only, size_t smem, cudaStream_t st) {
     const auto k = [&](auto kernel) {
@@ -1242,30 +1251,30 @@ cudaError_t launch_k_step(const Consts& c, const Dev& dv, const ClassPlan& cp, c
 cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, const Tile* tiles, const int* perm,
                         const StepIO& io, int observe_only, cudaStream_t st) {
     if (cp.n_tiles == 0) return cudaSuccess;
-    const bool ext = extended(c);
+    const int ext = extended(c);
     if (cp.ws && !observe_only)
-        return launch_overlapped(ext ? k_step_ws<true> : k_step_ws<false>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
+        return launch_overlapped(ext == 2 ? k_step_ws<2> : ext == 1 ? k_step_ws<1> : k_step_ws<0>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
                                  tiles + cp.tile_off,
                                  perm, io);
     const size_t smem = cp.W > 1 ? sizeof(float) * SMEM_PLANES * cp.block
                         : ext     ? 0
                                   : sizeof(float) * cp.block * (c.obs_dim + ROW_PAD);
     const Tile* t = tiles + cp.tile_off;
-    return ext ? launch_k_step<true>(c, dv, cp, t, perm, io, observe_only, smem, st)
-               : launch_k_step<false>(c, dv, cp, t, perm, io, observe_only, smem, st);
+    return ext == 2   ? launch_k_step<2>(c, dv, cp, t, perm, io, observe_only, smem, st)
+           : ext == 1 ? launch_k_step<1>(c, dv, cp, t, perm, io, observe_only, smem, st)
+                      : launch_k_step<0>(c, dv, cp, t, perm, io, observe_only, smem, st);
 }
 
-// The k_rollout instance for a handle: the general one, or without scenarios,
-// downwash and smooth contacts, and of those the single-drone one.
-const void* rollout_kernel(bool ext, bool single) {
-    if (ext) return (const void*)k_rollout<true, false>;
-    return single ? (const void*)k_rollout<false, true> : (const void*)k_rollout<false, false>;
+// The k_rollout instance for a handle (ext: extended()); of the common one, the
+// single-drone form where every env holds one drone.
+auto rollout_kernel(int ext, bool single) {
+    return ext == 2 ? k_rollout<2, false> : ext == 1 ? k_rollout<1, false> : single ? k_rollout<0, true> : k_rollout<0, false>;
 }
 
 // Its dynamic shared memory: two sets of staging planes and the CTA's
 // observation rows (none for single drones).
 size_t rollout_smem(const Consts& c, int block, bool single) {
-    const bool ext = extended(c);
+    const int ext = extended(c);
     return single && !ext ? 0 : sizeof(float) * block * (2 * SMEM_PLANES + (ext ? GOAL_STRIDE : 0) + c.obs_dim + ROW_PAD);
 }
 
@@ -1273,7 +1282,7 @@ int rollout_grid(const Consts& c, int block, bool single) {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const void* fn = rollout_kernel(extended(c), single);
+    const void* fn = (const void*)rollout_kernel(extended(c), single);
     const size_t smem = rollout_smem(c, block, single);
     allow_smem(fn, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
@@ -1283,10 +1292,9 @@ int rollout_grid(const Consts& c, int block, bool single) {
 cudaError_t launch_rollout_ws(const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int P, const int* perm,
                               const RolloutIO& io, int t0, int nsteps, cudaStream_t st) {
     if (n_tiles == 0) return cudaSuccess;
-    const bool ext = extended(c);
+    const int ext = extended(c);
     if (P != 1 && P != 2) return cudaErrorInvalidValue;
-    const auto k = P == 1 ? (ext ? k_rollout_ws<true, 1> : k_rollout_ws<false, 1>)
-                          : (ext ? k_rollout_ws<true, 2> : k_rollout_ws<false, 2>);
+    const auto k = P == 1 ? rollout_ws_kernel<1>(ext) : rollout_ws_kernel<2>(ext);
     return launch_overlapped(k, n_tiles, 64 * P, ws_smem(c, P), st, c, dv, tiles, perm, io, t0, nsteps);
 }
 
@@ -1294,11 +1302,11 @@ cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, in
                            int* counter, const RolloutIO& io, int t0, int nsteps, int grid, bool single,
                            cudaStream_t st) {
     const size_t smem = rollout_smem(c, block, single);
-    const cudaError_t e = allow_smem(rollout_kernel(extended(c), single), smem);
+    const cudaError_t e = allow_smem((const void*)rollout_kernel(extended(c), single), smem);
     if (e != cudaSuccess) return e;
     const int g = grid > 0 ? grid : n_tiles;
     const int grid_n = g < n_tiles ? g : n_tiles;
-    const auto k = extended(c) ? k_rollout<true, false> : single ? k_rollout<false, true> : k_rollout<false, false>;
+    const auto k = rollout_kernel(extended(c), single);
     return launch_overlapped(k, grid_n, block, smem, st, c, dv, tiles, n_tiles, perm, counter, io, t0, nsteps);
 }
 
