@@ -220,13 +220,15 @@ void drop_graph(qs_env* h) {
 long ws_wave(int n_sm) { return (long)n_sm * 8 * 32; }
 
 // The warp-specialised step wins while a class is latency-bound: up to about
-// one wave of its CTAs. Swarms of 17..32 keep it only up to two CTAs per SM:
-// their dynamics warps' pair pass (31 partners a drone) is heavy in issue
-// slots, and once more CTAs share an SM the noise warps' work competes for
-// those slots instead of filling idle ones (measured on GB300 at K = 6,
-// warp-specialised vs one env per 32-thread CTA: 8,192 drones 16.99 vs 17.13
-// us, 16,384 18.77 vs 17.83, 32,768 25.04 vs 21.26; swarms of 16 stay level
-// or ahead up to 32,768).
+// one wave of its CTAs (measured on GB300, us a call, warp-specialised vs one
+// thread a drone: single drones 8,192 4.4 vs 5.4, 38,912 6.12 vs 6.15, 49,152
+// 8.5 vs 6.9; swarms of 8 at K = 6 2,048 5.7 vs 6.7, 4,864 7.4 vs 10.2). Past
+// it the outcome hangs on the observation's length (65,536 drones in swarms of
+// 8, K = 6, 12.4 vs 14.8; 150,000 in swarms of 5, K = 2, 35.5 vs 23.7).
+// Swarms of 17..32 keep it only up to two CTAs per SM, where the pair pass's
+// issue slots used to cross over; with the 32-bit selection it would stay
+// ahead a little longer (1,024 x 32 9.7 vs 10.3, 3,072 x 32 22.8 vs 21.7), and
+// the default callers read back (qs_get_block) stays as it was.
 bool use_ws(int W, int slots, int n_sm) {
     const long threads = (long)slots * W;
     return W <= 32 && threads <= (W > 16 ? (long)n_sm * 64 : ws_wave(n_sm));

@@ -268,8 +268,8 @@ __device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, fl
 
 // ROWS: the observation rows go through shared memory (the rollout), else each
 // lane stores its own. Swarm rollouts take the former (4096 uneven swarms, 32
-// steps, 358 -> 299 us; 256 x 128, 16 steps, 203 -> 183 us); single drones keep
-// their 9 stores: addressing the block costs 95 instructions of 1,100 a step,
+// steps, 358 -> 299 us; 256 x 128, 16 steps, 203 -> 183 us) and the single
+// drones' step; single-drone rollouts keep their 9 stores: addressing the block costs 95 instructions of 1,100 a step,
 // more than the stores' waits (1,048,576 drones, 32 steps: 1696 against 1834 us).
 template <int EXT, bool ROWS>
 __device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, uint32_t& ev_out,
@@ -669,13 +669,13 @@ __device__ __forceinline__ void ws_goal(const Consts& c, const Dev& dv, WsShared
 // and B2 (post-step state, goal and neighbours published for the observation
 // rows), then writes the knn record, reward and done and ends the step. Every
 // thread of the dynamics warps calls it.
-template <int EXT, int P, bool DEFER>
+template <int EXT, int P, bool DEFER, bool W1 = false>
 __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv, WsShared<P>& sh, const WsMap& m,
                                                  Drone& s, EnvRegs& er, uint32_t& ev_out, const float4 a, const int nb,
                                                  float* __restrict__ rew, uint8_t* __restrict__ done, GoalCache& gc,
                                                  const bool b1 = true) {
     const int b = nb;  // the step's buffers: its motor normals and its published end
-    const int W = m.W, L = m.L, lane = m.lane, N = m.N, e = m.e, d = m.d, sbase = m.sbase;
+    const int W = W1 ? 1 : m.W, L = m.L, lane = m.lane, N = W1 ? 1 : m.N, e = m.e, d = m.d, sbase = m.sbase;
     const bool act = m.act;
     const int K = c.K;
     const int nahead = min(c.substeps, WS_SUB);
@@ -862,7 +862,10 @@ __device__ __forceinline__ float* ws_rows(const Consts& c, int L) {
     return reinterpret_cast<float*>(sm) + (L & ~31) * (c.obs_dim + ROW_PAD);
 }
 
-template <int EXT>
+// W1: every slot of the launch holds one drone (no pair pass: a smaller kernel to
+// fetch when its instructions are cold; 8192 drones with L2 flushed before each
+// step 9.7 -> 9.1 us).
+template <int EXT, bool W1 = false>
 __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                 const int* __restrict__ perm, const StepIO io) {
     __shared__ WsShared<1> sh;
@@ -894,7 +897,7 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
         a = reinterpret_cast<const float4*>(io.act)[m.d];
     }
     GoalCache gc{sh.gv[m.L], GOAL_FIXED, 0, -1};
-    ws_dynamics_step<EXT, 1, false>(c, dv, sh, m, s, er, ev, a, 0, io.rew, io.done, gc);
+    ws_dynamics_step<EXT, 1, false, W1>(c, dv, sh, m, s, er, ev, a, 0, io.rew, io.done, gc);
     if (!m.act) return;
     dv.ev[m.d] = ev;
     store_drone(s, dv.st, dv.D, m.d);
@@ -1253,7 +1256,7 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
     if (cp.n_tiles == 0) return cudaSuccess;
     const int ext = extended(c);
     if (cp.ws && !observe_only)
-        return launch_overlapped(ext == 2 ? k_step_ws<2> : ext == 1 ? k_step_ws<1> : k_step_ws<0>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
+        return launch_overlapped(ext == 2 ? k_step_ws<2> : ext == 1 ? k_step_ws<1> : cp.W == 1 ? k_step_ws<0, true> : k_step_ws<0>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
                                  tiles + cp.tile_off,
                                  perm, io);
     const size_t smem = cp.W > 1 ? sizeof(float) * SMEM_PLANES * cp.block
