@@ -590,8 +590,16 @@ struct WsShared {
     float gv[32 * P][GOAL_STRIDE];  // goal values of each lane's drone (GoalCache)
 };
 
-// Dynamic shared memory of a warp-specialised CTA: the noise side's rows.
+// Dynamic shared memory of a warp-specialised CTA: the noise side's rows. With
+// WsShared it passes the 48 KiB every kernel may have for 64 lanes and K = 8;
+// such a kernel asks for the most any shape needs.
 inline size_t ws_smem(const Consts& c, int P) { return sizeof(float) * 32 * P * (c.obs_dim + ROW_PAD); }
+inline cudaError_t allow_ws_smem(const void* fn, const Consts& c, int P) {
+    const size_t fixed = (P == 1 ? sizeof(WsShared<1>) : sizeof(WsShared<2>)) + 64;  // and a few words of the kernel's own
+    if (fixed + ws_smem(c, P) <= 48u << 10) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(sizeof(float) * 32 * P * (18 + 6 * QS_MAX_K + ROW_PAD)));
+}
 
 // Barrier among the P warps of one side (id 1: dynamics, id 2: noise); one
 // warp only needs its own lanes converged.
@@ -1187,6 +1195,8 @@ cudaError_t launch_serve(const Consts& c, const Dev& dv, const Tile* tiles, int 
     const int* pp = perm;
     int kk = k0;
     void* args[] = {&cc, &dd, &tt, &pp, &ii, &kk};
+    const cudaError_t e = allow_ws_smem(fn, c, P);
+    if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(fn, dim3(n_tiles), dim3(64 * P), args, ws_smem(c, P), st);
 }
 
@@ -1196,7 +1206,9 @@ int serve_resident_ctas(const Consts& c, int P) {
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int ext = extended(c);
     const void* fn = P == 1 ? serve_kernel<1>(ext) : serve_kernel<2>(ext);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess) return 0;
+    if (allow_ws_smem(fn, c, P) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess)
+        return 0;
     return occ * n_sm;
 }
 
@@ -1206,7 +1218,9 @@ int rollout_ws_resident_ctas(const Consts& c, int P) {
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     const int ext = extended(c);
     const void* fn = P == 1 ? (const void*)rollout_ws_kernel<1>(ext) : (const void*)rollout_ws_kernel<2>(ext);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess) return 0;
+    if (allow_ws_smem(fn, c, P) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, 64 * P, ws_smem(c, P)) != cudaSuccess)
+        return 0;
     return occ * n_sm;
 }
 
@@ -1298,6 +1312,8 @@ cudaError_t launch_rollout_ws(const Consts& c, const Dev& dv, const Tile* tiles,
     const int ext = extended(c);
     if (P != 1 && P != 2) return cudaErrorInvalidValue;
     const auto k = P == 1 ? rollout_ws_kernel<1>(ext) : rollout_ws_kernel<2>(ext);
+    const cudaError_t e = allow_ws_smem((const void*)k, c, P);
+    if (e != cudaSuccess) return e;
     return launch_overlapped(k, n_tiles, 64 * P, ws_smem(c, P), st, c, dv, tiles, perm, io, t0, nsteps);
 }
 
