@@ -1110,8 +1110,12 @@ __device__ __forceinline__ unsigned long long serve_wait(unsigned long long* go,
 // by the noise side after B2 and the next step's normals drawn after them,
 // then B3, after which thread 0 fences the CTA's host writes at system scope
 // and counts the CTA done; the last CTA publishes fin = k0 + k + 1.
+// The launch bound is how many CTAs an SM holds, and with it the largest handle
+// qs_serve_begin accepts: a scheduler takes three warps of up to 168 registers.
+// Left to itself the 64-lane common instance takes 193, two CTAs an SM; held to
+// three it fits in 144 without a spill (the general ones take 208 and 226).
 template <int EXT, int P>
-__global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_serve(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
+__global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : EXT == 0 ? 3 : 2)) k_serve(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                                   const int* __restrict__ perm, const ServeIO io, const int k0) {
     __shared__ WsShared<P> sh;
     __shared__ unsigned long long s_go;
