@@ -22,6 +22,18 @@ using namespace qsk;
 
 static thread_local std::string g_create_error;
 
+// What the launches of a captured rollout were made from: a graph is replayed
+// only for a call with the same. io.bulk is part of it, as an address may come
+// back as another kind of memory.
+struct GraphKey {
+    int T, fuse, block;
+    RolloutIO io;
+    bool operator==(const GraphKey& k) const {
+        return T == k.T && fuse == k.fuse && block == k.block && io.act == k.io.act && io.obs == k.io.obs &&
+               io.rew == k.io.rew && io.done == k.io.done && io.bulk == k.io.bulk;
+    }
+};
+
 struct qs_env {
     qs_config cfg{};
     cudaStream_t stream = nullptr;
@@ -55,10 +67,7 @@ struct qs_env {
     int use_graph = 1;
     int* d_counter = nullptr;
     cudaGraphExec_t graph = nullptr;
-    struct {
-        int T, fuse, block;
-        const void *a, *o, *r, *d;
-    } graph_key{};
+    GraphKey graph_key{};
     // device staging of qs_step_host (one allocation, made on first use)
     char* stage = nullptr;
     size_t st_obs = 0, st_rew = 0, st_done = 0;
@@ -769,19 +778,17 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
     if (!actions_dev || !aligned(actions_dev, 16)) return fail(h, QS_ERR_ARG, "qs_rollout: actions_dev NULL or misaligned");
     if (obs_dev && !aligned(obs_dev, 8)) return fail(h, QS_ERR_ARG, "qs_rollout: obs_dev must be 8-byte aligned");
     DeviceGuard g(h->device);
-    // Graph replay: the launches of one (T, buffers, shape) are captured once
-    // and replayed; any change of buffers or shape re-captures. The legacy
-    // default stream cannot be captured, so it launches directly.
-    if (!h->use_graph || h->stream == nullptr)
-        return enqueue_rollout(h, T, RolloutIO{actions_dev, obs_dev, reward_dev, done_dev, device_memory(obs_dev)});
-    const auto& k = h->graph_key;
-    if (h->graph && k.T == T && k.fuse == h->rollout_fuse && k.block == h->rollout_block && k.a == actions_dev &&
-        k.o == obs_dev && k.r == reward_dev && k.d == done_dev) {
+    const RolloutIO io{actions_dev, obs_dev, reward_dev, done_dev, device_memory(obs_dev)};
+    // Graph replay: the launches of one GraphKey are captured once and
+    // replayed; any change of it re-captures. The legacy default stream cannot
+    // be captured, so it launches directly.
+    if (!h->use_graph || h->stream == nullptr) return enqueue_rollout(h, T, io);
+    const GraphKey key{T, h->rollout_fuse, h->rollout_block, io};
+    if (h->graph && h->graph_key == key) {
         cudaError_t e = cudaGraphLaunch(h->graph, h->stream);
         return e == cudaSuccess ? QS_OK : cuda_fail(h, e, "rollout graph launch");
     }
     drop_graph(h);
-    const RolloutIO io{actions_dev, obs_dev, reward_dev, done_dev, device_memory(obs_dev)};
     cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return cuda_fail(h, e, "rollout capture begin");
     qs_status s = enqueue_rollout(h, T, io);
@@ -798,7 +805,7 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
         h->graph = nullptr;
         return cuda_fail(h, e, "rollout graph instantiate");
     }
-    h->graph_key = {T, h->rollout_fuse, h->rollout_block, actions_dev, obs_dev, reward_dev, done_dev};
+    h->graph_key = key;
     e = cudaGraphLaunch(h->graph, h->stream);
     return e == cudaSuccess ? QS_OK : cuda_fail(h, e, "rollout graph launch");
 }
