@@ -292,8 +292,9 @@ qs_status qs_serve_end(qs_env* h);
  * (largest swarms first) and keep each drone's state in registers across the
  * steps of a launch. The T steps run as ceil(T / fuse) launches (see
  * qs_set_rollout_shape). On a non-default stream the launches are captured
- * into a CUDA graph on the first call and replayed while T, the buffers and
- * the shape stay the same. Not callable during a caller's own stream capture
+ * into a CUDA graph on the first call and replayed while T, the buffers (and
+ * their kind of memory), the shape and the seed of the last full reset stay the
+ * same. Not callable during a caller's own stream capture
  * when a (re)capture is needed. */
 qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_dev, float* reward_dev,
                      uint8_t* done_dev);

@@ -24,13 +24,16 @@ static thread_local std::string g_create_error;
 
 // What the launches of a captured rollout were made from: a graph is replayed
 // only for a call with the same. io.bulk is part of it, as an address may come
-// back as another kind of memory.
+// back as another kind of memory, and so are the Philox keys, which a full
+// reset changes.
 struct GraphKey {
     int T, fuse, block;
+    uint32_t key0, key1;
     RolloutIO io;
     bool operator==(const GraphKey& k) const {
-        return T == k.T && fuse == k.fuse && block == k.block && io.act == k.io.act && io.obs == k.io.obs &&
-               io.rew == k.io.rew && io.done == k.io.done && io.bulk == k.io.bulk;
+        return T == k.T && fuse == k.fuse && block == k.block && key0 == k.key0 && key1 == k.key1 &&
+               io.act == k.io.act && io.obs == k.io.obs && io.rew == k.io.rew && io.done == k.io.done &&
+               io.bulk == k.io.bulk;
     }
 };
 
@@ -783,7 +786,7 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
     // replayed; any change of it re-captures. The legacy default stream cannot
     // be captured, so it launches directly.
     if (!h->use_graph || h->stream == nullptr) return enqueue_rollout(h, T, io);
-    const GraphKey key{T, h->rollout_fuse, h->rollout_block, io};
+    const GraphKey key{T, h->rollout_fuse, h->rollout_block, h->c.key0, h->c.key1, io};
     if (h->graph && h->graph_key == key) {
         cudaError_t e = cudaGraphLaunch(h->graph, h->stream);
         return e == cudaSuccess ? QS_OK : cuda_fail(h, e, "rollout graph launch");

@@ -63,3 +63,18 @@ def test_replayed_rollout_follows_the_kind_of_its_buffer(api, handle):
         assert api.qs_rollout(handle, 3, act, obs, None, None) == 0
         seen.append((api.fake_captures() - before, api.fake_bulk()))
     assert seen == [(1, 1), (0, 1), (1, 0), (0, 0), (0, 0), (1, 1)]
+
+
+def test_replayed_rollout_follows_the_seed(api, handle):
+    """A captured launch holds the Philox keys; a full reset that changes them is
+    captured again, the same seed or a masked reset is not."""
+    keep, act, obs = buffers()
+    mask = (C.c_uint8 * 4)(1, 0, 0, 1)
+    seen = []
+    for seed, masked in ((None, False), (5, False), (5, False), (6, True), (5 + (1 << 32), False), (None, False)):
+        if seed is not None:
+            assert api.qs_reset(handle, seed, C.addressof(mask) if masked else None, None) == 0
+        before = api.fake_captures()
+        assert api.qs_rollout(handle, 3, act, obs, None, None) == 0
+        seen.append(api.fake_captures() - before)
+    assert seen == [1, 1, 0, 0, 1, 0]
