@@ -110,7 +110,10 @@ qs_status busy(qs_env* h, const char* who) {
     return fail(h, QS_ERR_ARG, std::string(who) + ": the handle is serving (call qs_serve_end first)");
 }
 
+// Reports a failed CUDA call, and takes the error it left with the runtime: the
+// launches that check for one (cudaGetLastError) would report it as theirs.
 qs_status cuda_fail(qs_env* h, cudaError_t e, const char* where) {
+    cudaGetLastError();
     return fail(h, QS_ERR_CUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
@@ -799,6 +802,7 @@ qs_status qs_rollout(qs_env* h, int32_t T, const float* actions_dev, float* obs_
     e = cudaStreamEndCapture(h->stream, &graph);
     if (s != QS_OK) {
         if (graph) cudaGraphDestroy(graph);
+        cudaGetLastError();  // of the capture that the failed launch invalidated
         return s;
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "rollout capture end");

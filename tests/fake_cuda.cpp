@@ -13,7 +13,7 @@
 namespace {
 cudaError_t g_last = cudaSuccess, g_next_launch = cudaSuccess;
 std::map<const void*, int> g_kind;  // pointers with a kind of memory of their own (else device memory)
-bool g_capturing = false;
+bool g_capturing = false, g_invalid = false;  // a failed launch invalidates the capture
 int g_captures = 0, g_replays = 0, g_bulk = -1;
 
 cudaError_t ret(cudaError_t e) {
@@ -23,6 +23,7 @@ cudaError_t ret(cudaError_t e) {
 cudaError_t launch() {  // fails once after fake_fail_next_launch
     const cudaError_t e = g_next_launch;
     g_next_launch = cudaSuccess;
+    g_invalid |= g_capturing && e != cudaSuccess;
     return ret(e);
 }
 cudaError_t rollout(const qsk::RolloutIO& io) {
@@ -76,13 +77,14 @@ cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* s) {
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
     g_capturing = true;
+    g_invalid = false;
     ++g_captures;
     return cudaSuccess;
 }
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
     g_capturing = false;
-    *g = (cudaGraph_t)(size_t)g_captures;
-    return cudaSuccess;
+    *g = g_invalid ? nullptr : (cudaGraph_t)(size_t)g_captures;
+    return g_invalid ? ret(cudaErrorStreamCaptureInvalidated) : cudaSuccess;
 }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long) { *e = (cudaGraphExec_t)g; return cudaSuccess; }
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }

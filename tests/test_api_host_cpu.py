@@ -78,3 +78,16 @@ def test_replayed_rollout_follows_the_seed(api, handle):
         assert api.qs_rollout(handle, 3, act, obs, None, None) == 0
         seen.append(api.fake_captures() - before)
     assert seen == [1, 1, 0, 0, 1, 0]
+
+
+def test_a_failed_launch_is_reported_once(api, handle):
+    """The error a failed launch leaves with the runtime is taken by the call that
+    reports it: later calls, whose launches check for one, must not find it."""
+    keep, act, obs = buffers()
+    calls = [lambda: api.qs_step(handle, act, obs, None, None), lambda: api.qs_rollout(handle, 2, act, obs, None, None),
+             lambda: api.qs_reset(handle, 3, None, None)]
+    for call in calls:
+        api.fake_fail_next_launch(1)
+        assert call() != 0
+        assert api.fake_pending_error() == 0
+        assert call() == 0
