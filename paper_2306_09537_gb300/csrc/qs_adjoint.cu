@@ -362,7 +362,7 @@ __device__ __forceinline__ void smooth_substep(const Consts& c, Drone& s, const 
     if (act) sp[lt] = make_float4(s.x[0], s.x[1], s.x[2], 0.f);
     group_sync(bid, bn);
     float pa[3] = {0.f, 0.f, 0.f};
-    if (act) pair_acc(c, s.x, sp, sbase, lane, N, p.arm, pa);
+    if (act && N > 1) pair_acc(c, s.x, sp, sbase, lane, N, p.arm, pa);
     group_sync(bid, bn);
     if (act) substep<false, 1>(s, p, c, u, tick, d, sub, pa, nrm);
 }
@@ -612,7 +612,7 @@ __global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_d
                         sla[2 * nt + lt] = la[2];
                     }
                     group_sync(bid, nb);
-                    if (act) pair_vjp(c, si.x, la, sp, sla, nt, sbase, lane, N, p.arm, lx);
+                    if (act && N > 1) pair_vjp(c, si.x, la, sp, sla, nt, sbase, lane, N, p.arm, lx);
                     group_sync(bid, nb);
                 }
                 if (act) {

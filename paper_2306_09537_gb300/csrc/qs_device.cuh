@@ -484,7 +484,9 @@ __device__ __forceinline__ float pair_far_d2(float arm, float inv_beta) {
 // Calls body(j), in increasing j, for every partner j of the thread's drone with
 // d2(j) between 0 and far2 (pair_far_d2). Most swarms have no such pair in most
 // substeps, so the distances of 32 partners are tested first, four at a time
-// and without a branch between them, and only the near ones are visited.
+// and without a branch between them, and only the near ones are visited. Callers
+// leave out a drone without partners (four distances a substep for nothing:
+// 40,000 single drones, gradients of 24 steps 395 -> 358 us).
 template <class D2, class Body>
 __device__ __forceinline__ void near_pairs(int lane, int N, float far2, const D2& d2, const Body& body) {
     for (int j0 = 0; j0 < N; j0 += 32) {
