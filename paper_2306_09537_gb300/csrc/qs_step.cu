@@ -498,7 +498,8 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
     // the commands of step t + 1 are loaded while step t computes, so their
     // HBM latency leaves each step's dependent chain
     float4 a_next = m.act ? *(act4 + (size_t)t0 * D) : make_float4(0.f, 0.f, 0.f, 0.f);
-    float* goals = reinterpret_cast<float*>(sm + 2 * SMEM_PLANES / 4 * blockDim.x);  // the general instance's goal values
+    // the general instances' goal values, after the staging planes
+    float* goals = reinterpret_cast<float*>(sm + (W1 ? 0 : 2 * SMEM_PLANES / 4 * blockDim.x));
     GoalCache gc{goals + GOAL_STRIDE * threadIdx.x, GOAL_FIXED, 0, -1};
     const RowMap rm = W1 ? RowMap() : map_rows(m.act, m.d, W, c.obs_dim);
     float* rows = goals + (EXT ? GOAL_STRIDE * blockDim.x : 0) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
@@ -521,8 +522,8 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
 // Persistent rollout: CTAs take tiles from *counter until none is left; every
 // CTA draws one number past the tiles, and the last of those puts the counter
 // back to zero for the next launch (a memset before each launch cost a launch
-// of its own). Tiles are ordered costliest first. The W1 instance
-// (EXT = 0 only) serves handles whose envs all hold one drone: 107
+// of its own). Tiles are ordered costliest first. The W1 instances (EXT = 0
+// and 2) serve handles whose envs all hold one drone: for EXT = 0 107
 // registers instead of 121 and no untaken swarm code in the step loop (with
 // the smooth contacts compiled out of the EXT = 0 instances, batched
 // 1,048,576 single-drone envs went from 1.75e10 to 1.90e10 quadrotor-steps/s,
@@ -530,8 +531,11 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
 // spill, five warps a scheduler instead of four (1,048,576 drones, 32 steps,
 // 1687 -> 1632 us, in 32-thread CTAs 1593; at 88 registers 1644). Swarms spill
 // below 128 (16,384 x 8, 64 steps: 128 registers 746 us, 112 799, 160 901).
+// With smooth contacts the rows' way through shared memory cost single drones
+// 8% (34,000 drones, 32 steps: 102 us before the rows went that way, 111 after,
+// 96 in this instance, whose lanes store their own; 300,000 drones 579, 589, 532).
 template <int EXT, bool W1>
-__global__ void __maxnreg__(W1 ? 104 : 128) k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
+__global__ void __maxnreg__(W1 && !EXT ? 104 : 128) k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                        const int n_tiles, const int* __restrict__ perm,
                                                        int* __restrict__ counter, const RolloutIO io, const int t0,
                                                        const int nsteps) {
@@ -1286,17 +1290,18 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
                       : launch_k_step<0>(c, dv, cp, t, perm, io, observe_only, smem, st);
 }
 
-// The k_rollout instance for a handle (ext: extended()); of the common one, the
-// single-drone form where every env holds one drone.
+// The k_rollout instance for a handle (ext: extended()); of the common and the
+// smooth one, the single-drone form where every env holds one drone.
 auto rollout_kernel(int ext, bool single) {
-    return ext == 2 ? k_rollout<2, false> : ext == 1 ? k_rollout<1, false> : single ? k_rollout<0, true> : k_rollout<0, false>;
+    if (ext == 2) return single ? k_rollout<2, true> : k_rollout<2, false>;
+    return ext == 1 ? k_rollout<1, false> : single ? k_rollout<0, true> : k_rollout<0, false>;
 }
 
-// Its dynamic shared memory: two sets of staging planes and the CTA's
-// observation rows (none for single drones).
+// Its dynamic shared memory: goal values (general instances) and, but for the
+// single-drone forms, two sets of staging planes and the CTA's observation rows.
 size_t rollout_smem(const Consts& c, int block, bool single) {
-    const int ext = extended(c);
-    return single && !ext ? 0 : sizeof(float) * block * (2 * SMEM_PLANES + (ext ? GOAL_STRIDE : 0) + c.obs_dim + ROW_PAD);
+    const int ext = extended(c), goal = ext ? GOAL_STRIDE : 0;
+    return sizeof(float) * block * (single && ext != 1 ? goal : 2 * SMEM_PLANES + goal + c.obs_dim + ROW_PAD);
 }
 
 int rollout_grid(const Consts& c, int block, bool single) {
