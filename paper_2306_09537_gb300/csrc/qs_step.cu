@@ -269,8 +269,9 @@ __device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, fl
 // ROWS: the observation rows go through shared memory (the rollout), else each
 // lane stores its own. Swarm rollouts take the former (4096 uneven swarms, 32
 // steps, 358 -> 299 us; 256 x 128, 16 steps, 203 -> 183 us) and the single
-// drones' step; single-drone rollouts keep their 9 stores: addressing the block costs 95 instructions of 1,100 a step,
-// more than the stores' waits (1,048,576 drones, 32 steps: 1696 against 1834 us).
+// drones' step; single-drone rollouts with short rows keep their stores (9 at
+// K = 0): addressing the block costs 95 instructions of 1,100 a step, more than
+// the stores' waits (1,048,576 drones, 32 steps: 1696 against 1834 us; single_form).
 template <int EXT, bool ROWS>
 __device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, uint32_t& ev_out,
                                           float4* sp, float* sv, const bool act, const int lane, const int N,
@@ -523,7 +524,7 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
 // CTA draws one number past the tiles, and the last of those puts the counter
 // back to zero for the next launch (a memset before each launch cost a launch
 // of its own). Tiles are ordered costliest first. The W1 instances (EXT = 0
-// and 2) serve handles whose envs all hold one drone: for EXT = 0 107
+// and 2) serve handles whose envs all hold one drone (single_form): for EXT = 0 107
 // registers instead of 121 and no untaken swarm code in the step loop (with
 // the smooth contacts compiled out of the EXT = 0 instances, batched
 // 1,048,576 single-drone envs went from 1.75e10 to 1.90e10 quadrotor-steps/s,
@@ -1290,25 +1291,37 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
                       : launch_k_step<0>(c, dv, cp, t, perm, io, observe_only, smem, st);
 }
 
-// The k_rollout instance for a handle (ext: extended()); of the common and the
-// smooth one, the single-drone form where every env holds one drone.
-auto rollout_kernel(int ext, bool single) {
-    if (ext == 2) return single ? k_rollout<2, true> : k_rollout<2, false>;
-    return ext == 1 ? k_rollout<1, false> : single ? k_rollout<0, true> : k_rollout<0, false>;
+// Whether a handle's rollout takes the single-drone form of its instance (the
+// common and the smooth one have it): every env holds one drone, and the row is
+// short, so that its lane had better store it than send it through shared memory.
+// Measured with one drone an env and K neighbour fields, us, stored by the lane
+// against sent: common 30,000 drones, 16 steps K = 1 47 and 54, K = 2 51 and 55,
+// K = 6 81 and 58; 100,000, 12 steps K = 2 115 and 92, K = 6 270 and 96; smooth
+// 30,000 K = 2 54 and 61, 100,000 K = 1 91 and 106, K = 6 245 and 112.
+bool single_form(const Consts& c, bool single) { return single && extended(c) != 1 && c.K <= 2; }
+
+// The k_rollout instance for a handle.
+auto rollout_kernel(const Consts& c, bool single) {
+    const bool form = single_form(c, single);
+    switch (extended(c)) {
+        case 2: return form ? k_rollout<2, true> : k_rollout<2, false>;
+        case 1: return k_rollout<1, false>;
+        default: return form ? k_rollout<0, true> : k_rollout<0, false>;
+    }
 }
 
 // Its dynamic shared memory: goal values (general instances) and, but for the
 // single-drone forms, two sets of staging planes and the CTA's observation rows.
 size_t rollout_smem(const Consts& c, int block, bool single) {
-    const int ext = extended(c), goal = ext ? GOAL_STRIDE : 0;
-    return sizeof(float) * block * (single && ext != 1 ? goal : 2 * SMEM_PLANES + goal + c.obs_dim + ROW_PAD);
+    const int goal = extended(c) ? GOAL_STRIDE : 0;
+    return sizeof(float) * block * (single_form(c, single) ? goal : 2 * SMEM_PLANES + goal + c.obs_dim + ROW_PAD);
 }
 
 int rollout_grid(const Consts& c, int block, bool single) {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const void* fn = (const void*)rollout_kernel(extended(c), single);
+    const void* fn = (const void*)rollout_kernel(c, single);
     const size_t smem = rollout_smem(c, block, single);
     allow_smem(fn, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
@@ -1330,11 +1343,11 @@ cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, in
                            int* counter, const RolloutIO& io, int t0, int nsteps, int grid, bool single,
                            cudaStream_t st) {
     const size_t smem = rollout_smem(c, block, single);
-    const cudaError_t e = allow_smem((const void*)rollout_kernel(extended(c), single), smem);
+    const auto k = rollout_kernel(c, single);
+    const cudaError_t e = allow_smem((const void*)k, smem);
     if (e != cudaSuccess) return e;
     const int g = grid > 0 ? grid : n_tiles;
     const int grid_n = g < n_tiles ? g : n_tiles;
-    const auto k = rollout_kernel(extended(c), single);
     return launch_overlapped(k, grid_n, block, smem, st, c, dv, tiles, n_tiles, perm, counter, io, t0, nsteps);
 }
 
