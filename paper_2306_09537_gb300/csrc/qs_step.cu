@@ -447,7 +447,7 @@ __device__ __forceinline__ SlotMap map_slot(const Dev& dv, const Tile& tile, con
 // drones 10.3 -> 8.0 us a step, 262,144 28.7 -> 28.3); past them every CTA's
 // wait costs more than the launch (1,048,576: 83.2 -> 87.9 us).
 constexpr int STEP_OVERLAP_WAVES = 2;
-template <int W, int EXT, bool OVERLAP = true>
+template <int W, int EXT, bool OVERLAP = true, bool ROWS = (W == 1 && !EXT)>
 __global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                     const int* __restrict__ perm, const StepIO io, const int observe_only) {
     extern __shared__ float4 sm[];
@@ -464,9 +464,9 @@ __global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(con
                                               : make_float4(0.f, 0.f, 0.f, 0.f);
     float gv[GOAL_VALUES];
     GoalCache gc{gv, GOAL_FIXED, 0, -1};
-    // single drones: rows of a warp as one block (see RowMap; 65,536 drones 8.0 ->
-    // 7.7 us, 1,048,576 83.3 -> 82.5 us)
-    constexpr bool ROWS = W == 1 && !EXT;
+    // single drones: rows of a warp as one block (see RowMap; 150,000 drones 15.6 ->
+    // 13.5 us, 300,000 28.9 -> 26.0; from 600,000 on the state's traffic is what
+    // counts: 1,048,576 81.0 and 80.5), or stored by the lanes (lane_rows)
     const RowMap rm = ROWS ? map_rows(m.act, m.d, 1, c.obs_dim) : RowMap();
     float* rows = reinterpret_cast<float*>(sm) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
     step_body<EXT, ROWS>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
@@ -1248,6 +1248,15 @@ int step_wave(int block) {
     return n_sm * (768 / block);
 }
 
+// Whether the lanes of the large single-drone step store their own rows. Held to
+// 80 registers, the form that sends them spills twice the bytes, which its
+// substeps load again: it pays while the rows weigh more than the substeps.
+// Measured, us a step of 1,048,576 drones at K = 0, stored by the lane against
+// sent: 2 substeps 81.0 and 80.5 (300,000 drones 28.9 and 25.9), 3 90.4 and 92.2,
+// 4 103.0 and 107.0, 6 139.5 and 143.5; 600,000 drones at K = 1: 4 substeps 67.1
+// and 67.4, 6 86.4 and 89.0.
+bool lane_rows(const Consts& c) { return c.substeps > 2 + 2 * c.K; }
+
 template <int EXT>
 cudaError_t launch_k_step(const Consts& c, const Dev& dv, const ClassPlan& cp, const Tile* t, const int* perm,
                           const StepIO& io, int observe_only, size_t smem, cudaStream_t st) {
@@ -1260,7 +1269,10 @@ cudaError_t launch_k_step(const Consts& c, const Dev& dv, const ClassPlan& cp, c
             if (e == cudaSuccess) e = allow_smem((const void*)k_step<1, EXT, false>, smem);
             if (e != cudaSuccess) return e;
             if (cp.n_tiles <= STEP_OVERLAP_WAVES * step_wave(cp.block)) return k(k_step<1, EXT>);
-            k_step<1, EXT, false><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only);
+            if (lane_rows(c))
+                k_step<1, EXT, false, false><<<cp.n_tiles, cp.block, 0, st>>>(c, dv, t, perm, io, observe_only);
+            else
+                k_step<1, EXT, false><<<cp.n_tiles, cp.block, smem, st>>>(c, dv, t, perm, io, observe_only);
             return cudaGetLastError();
         }
         case 2: return k(k_step<2, EXT>);
