@@ -5,13 +5,14 @@ import pytest
 import torch
 
 from gpu_helpers import DEV
+from paper_2306_09537_gb300 import qs
 from paper_2306_09537_gb300.env import QuadSwarmEnv
 
 pytestmark = pytest.mark.gpu
 FEATS = ("floor", "walls", "motor_noise", "obs_noise", "dr", "collisions", "auto_reset")
 
 
-@pytest.mark.parametrize("sizes,K", [([1] * 3000, 0), ([8] * 300, 6), ([1, 4, 9, 33] * 8, 2), ([64] * 20, 6)])
+@pytest.mark.parametrize("sizes,K", [([1] * 3000, 0), ([1] * 45000, 1), ([8] * 300, 6), ([1, 4, 9, 33] * 8, 2), ([64] * 20, 6)])
 def test_captured_closed_loop_with_a_side_stream(sizes, K):
     main, side = torch.cuda.Stream(), torch.cuda.Stream()
 
@@ -53,3 +54,24 @@ def test_captured_closed_loop_with_a_side_stream(sizes, K):
         assert torch.equal(logs[0], logs[1])
         for p, q in ((a, c), (b, d)):
             assert torch.equal(p.obs, q.obs) and torch.equal(p.reward, q.reward)
+
+
+@pytest.mark.parametrize("sizes,K", [([1] * 40000, 3), ([8] * 300, 6), ([1, 4, 9, 33] * 8, 2)])
+def test_captured_rollout_without_its_own_graph(sizes, K):
+    s = torch.cuda.Stream()
+    with torch.cuda.stream(s):
+        a, b = (QuadSwarmEnv(len(sizes), sizes, K, FEATS, seed=5, device=DEV, stream=s) for _ in range(2))
+        acts = torch.rand(4, a.D, 4, generator=torch.Generator(device=DEV).manual_seed(1), device=DEV)
+        rows = [torch.empty(4, a.D, a.obs_dim, device=DEV) for _ in range(2)]
+        for env in (a, b):
+            qs.qs_set_rollout_shape(env.h, qs.qs_get_rollout_shape(env.h)[0], 3, False)
+        s.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            a.rollout(acts * 0.5, rows[0])
+            a.rollout(acts, rows[0])
+        g.replay()
+        b.rollout(acts * 0.5, rows[1])
+        b.rollout(acts, rows[1])
+        s.synchronize()
+        assert torch.equal(rows[0], rows[1])
