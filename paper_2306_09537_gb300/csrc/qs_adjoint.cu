@@ -345,10 +345,12 @@ __device__ __forceinline__ bool group_sync_or(int id, int n, bool v) {
     // barrier numbers as immediates: with a number in a register the CTA is
     // given all 16, and an SM's 64 then hold 4 CTAs
     if (id == 1)
-        asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+        asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 1, %2, p;\n"
+                     " selp.u32 %0, 1, 0, q;\n}"
                      : "=r"(r) : "r"((uint32_t)v), "r"(n) : "memory");
     else
-        asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 2, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+        asm volatile("{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.red.or.pred q, 2, %2, p;\n"
+                     " selp.u32 %0, 1, 0, q;\n}"
                      : "=r"(r) : "r"((uint32_t)v), "r"(n) : "memory");
     return r != 0;
 }
@@ -505,8 +507,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
 // DENSE: 64-thread CTAs held to 168 registers (a few spills), six an SM
 // instead of four, for batches of several waves (dense_backward()).
 template <bool DENSE>
-__global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_diff_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
-                                                            const int* __restrict__ perm, const DiffArgs a) {
+__global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1)
+    k_diff_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles, const int* __restrict__ perm, const DiffArgs a) {
     extern __shared__ float4 sm4[];
     float* sm = reinterpret_cast<float*>(sm4);
     const int nb = blockDim.x >> 1, grp = threadIdx.x >= nb ? 1 : 0, lt = threadIdx.x - grp * nb, bid = 1 + grp;
@@ -1256,8 +1258,8 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diffd_fwd(const Consts c, con
 // each step's pre-collision state) into one scratch buffer while group 1
 // reverses segment s from the other.
 template <bool ET, bool DENSE>
-__global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_diffd_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
-                                                             const int* __restrict__ perm, const DiffArgs a) {
+__global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1)
+    k_diffd_bwd(const Consts c, const Dev dv, const Tile* __restrict__ tiles, const int* __restrict__ perm, const DiffArgs a) {
     extern __shared__ float4 sm4[];
     float* sm = reinterpret_cast<float*>(sm4);
     const int nb = blockDim.x >> 1, grp = threadIdx.x >= nb ? 1 : 0, lt = threadIdx.x - grp * nb, bid = 1 + grp;
@@ -1282,7 +1284,8 @@ __global__ void __launch_bounds__(DENSE ? 64 : ADJ_BLOCK_MAX, DENSE ? 6 : 1) k_d
     // RFLAG_BITS are taken as responding); the reverse skips the collision
     // adjoint of a step without responses, which is then the identity
     uint32_t* rflag = reinterpret_cast<uint32_t*>(sm + BWD_PLANES * nb);
-    const int S = c.substeps, S1 = c.substeps + 1;  // saved states per step: each substep's input, then the pre-collision state
+    // saved states per step: each substep's input, then the pre-collision state
+    const int S = c.substeps, S1 = c.substeps + 1;
     const size_t sbuf = (size_t)a.C * S1 * NSUB * D;  // floats of one scratch buffer
     Prm p;
     float g[3] = {0.f, 0.f, 0.f};

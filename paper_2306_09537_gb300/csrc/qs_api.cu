@@ -190,7 +190,7 @@ void build_tiles(qs_env* h, std::vector<Tile>& tiles) {
         cp.tile_off = (int)tiles.size();
         cp.n_tiles = 0;
         for (int s = 0; s < h->class_slots[ci]; s += per) {
-            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), cp.W, 0});
+            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), cp.W});
             ++cp.n_tiles;
         }
     }
@@ -205,7 +205,7 @@ void build_rollout_tiles(qs_env* h, std::vector<Tile>& tiles, int block) {
         const int W = h->plan[ci].W;
         const int per = block / W;
         for (int s = 0; s < h->class_slots[ci]; s += per)
-            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), W, 0});
+            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), W});
     }
 }
 
@@ -221,7 +221,7 @@ void build_ws_tiles(qs_env* h, std::vector<Tile>& tiles) {
     for (size_t ci = 0; ci < h->plan.size(); ++ci) {
         const int W = h->plan[ci].W, per = 32 * h->ws_p / W;
         for (int s = 0; s < h->class_slots[ci]; s += per)
-            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), W, 0});
+            tiles.push_back(Tile{h->class_first_slot[ci] + s, std::min(per, h->class_slots[ci] - s), W});
     }
 }
 
@@ -240,10 +240,11 @@ long ws_wave(int n_sm) { return (long)n_sm * 8 * 32; }
 // 8.5 vs 6.9; swarms of 8 at K = 6 2,048 5.7 vs 6.7, 4,864 7.4 vs 10.2). Past
 // it the outcome hangs on the observation's length (65,536 drones in swarms of
 // 8, K = 6, 12.4 vs 14.8; 150,000 in swarms of 5, K = 2, 35.5 vs 23.7).
-// Swarms of 17..32 keep it only up to two CTAs per SM, where the pair pass's
-// issue slots used to cross over; with the 32-bit selection it would stay
-// ahead a little longer (1,024 x 32 9.7 vs 10.3, 3,072 x 32 22.8 vs 21.7), and
-// the default callers read back (qs_get_block) stays as it was.
+// Swarms of 17..32 keep it only up to two CTAs per SM. The lines lie where the
+// two crossed over with the 64-bit neighbour selection; with the 32-bit one the
+// warp-specialised step is ahead a little longer (1,024 x 32 9.7 vs 10.3, 3,072
+// x 32 22.8 vs 21.7), so a few sizes past either line would gain from asking for
+// it (qs_set_block). A rule that also looks at K is not there yet.
 bool use_ws(int W, int slots, int n_sm) {
     const long threads = (long)slots * W;
     return W <= 32 && threads <= (W > 16 ? (long)n_sm * 64 : ws_wave(n_sm));

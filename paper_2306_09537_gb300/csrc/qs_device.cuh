@@ -317,7 +317,7 @@ __device__ __forceinline__ bool qs_check(int32_t*, bool) { return true; }
 __device__ __forceinline__ Tile tile_at(const Dev& dv, const Tile* __restrict__ tiles, int i, int lanes) {
     if (dv.uni_n) {
         const int per = lanes >> dv.uni_wlog, first = i * per;
-        return Tile{first, min(per, dv.E - first), 1 << dv.uni_wlog, 1};
+        return Tile{first, min(per, dv.E - first), 1 << dv.uni_wlog};
     }
     return tiles[i];
 }
@@ -384,9 +384,13 @@ __device__ __forceinline__ void comp_add_prod(float& hi, float& lo, float a, flo
 // A drone's state in memory: planes of float4 [D] that hold the 30 public floats
 // and, in the two that remain of the last, the low-order parts of w_x and w_y,
 // then a plane of float [D] with that of w_z: 132 bytes a drone (144 with a
-// ninth float4 plane for the low-order parts; a step of 1,048,576 single
-// drones, which memory bounds, 84.0 -> 83.3 us).
-__device__ __forceinline__ float* low_plane(float4* st, int D) { return reinterpret_cast<float*>(st + (size_t)NPLANE_PUBLIC * D); }
+// ninth float4 plane for the low-order parts). A step of 1,048,576 single drones
+// gains by it while they fly (82 -> 78 us soon after a reset, rows sent through
+// shared memory included) and hardly any once most lie on the floor or at the
+// walls (82.5 and 80.5, run to run 84): the same bytes, but longer substeps.
+__device__ __forceinline__ float* low_plane(float4* st, int D) {
+    return reinterpret_cast<float*>(st + (size_t)NPLANE_PUBLIC * D);
+}
 
 __device__ __forceinline__ void load_drone(Drone& s, float4* st, int D, int d) {
     float4 q[NPLANE];
@@ -524,7 +528,8 @@ __device__ __forceinline__ void pair_acc(const Consts& c, const float x[3], cons
         const float4 q = sp[sbase + j];
         const float r0 = x[0] - q.x, r1 = x[1] - q.y, r2 = x[2] - q.z;
         const float d = sqrtf(__fmaf_rn(r2, r2, __fmaf_rn(r1, r1, __fmul_rn(r0, r0))));
-        const float psi = __fmul_rn(__fmul_rn(kcg, softplus_b(__fsub_rn(2.f * arm, d), c.beta, c.inv_beta)), __frcp_rn(d));
+        const float sp_ = softplus_b(__fsub_rn(2.f * arm, d), c.beta, c.inv_beta);
+        const float psi = __fmul_rn(__fmul_rn(kcg, sp_), __frcp_rn(d));
         out[0] = fmaf(psi, r0, out[0]);
         out[1] = fmaf(psi, r1, out[1]);
         out[2] = fmaf(psi, r2, out[2]);
@@ -1056,7 +1061,8 @@ __device__ __forceinline__ bool pair_scan(const Consts& c, const Drone& s, float
         const auto word = [&](int j) {
             float dx, dy, dz;
             const float4 q = sp[j];
-            return (uint64_t)__float_as_uint(pair_key(s.x[0], s.x[1], s.x[2], q.x, q.y, q.z, dx, dy, dz)) << 32 | (uint32_t)j;
+            const float key = pair_key(s.x[0], s.x[1], s.x[2], q.x, q.y, q.z, dx, dy, dz);
+            return (uint64_t)__float_as_uint(key) << 32 | (uint32_t)j;
         };
         if (N <= 8) {
 #pragma unroll

@@ -98,7 +98,6 @@ struct Tile {
     int first;  // first slot (index into perm)
     int count;  // slots in this tile
     int W;      // width class of its slots
-    int pad;
 };
 
 struct ClassPlan {

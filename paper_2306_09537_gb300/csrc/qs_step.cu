@@ -34,7 +34,8 @@ constexpr int SMEM_PLANES = 8;
 // the padding of its block (RowMap)
 constexpr int ROW_PAD = 6;
 // and the most the kernels ask for
-constexpr int STEP_SMEM_MAX = (int)sizeof(float) * MAX_BLOCK * (2 * SMEM_PLANES + GOAL_STRIDE + 18 + 6 * QS_MAX_K + ROW_PAD);
+constexpr int STEP_SMEM_MAX =
+    (int)sizeof(float) * MAX_BLOCK * (2 * SMEM_PLANES + GOAL_STRIDE + 18 + 6 * QS_MAX_K + ROW_PAD);
 
 // The step kernels come in three instances, EXT = extended_instance(): 0 the
 // common configuration (one goal, no downwash, the paper's discrete contacts)
@@ -243,7 +244,8 @@ __device__ __forceinline__ void rows_free(const RowMap& r) {
 // Sends the warp's blocks on their way (every lane calls it): bulk copies, or
 // without bulk (destinations that may lie in host memory) stores by the lanes
 // that share a block, side by side.
-__device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, float* __restrict__ obs, int od, bool bulk) {
+__device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, float* __restrict__ obs, int od,
+                                          bool bulk) {
     const int sh = row_shift(r, obs, od);
     const int n = r.n * od - sh, m = n & ~3;  // floats past the 8 bytes before the units
     const float* src = rows + r.off + sh;
@@ -273,11 +275,12 @@ __device__ __forceinline__ void send_rows(const RowMap& r, const float* rows, fl
 // K = 0): addressing the block costs 95 instructions of 1,100 a step, more than
 // the stores' waits (1,048,576 drones, 32 steps: 1696 against 1834 us; single_form).
 template <int EXT, bool ROWS>
-__device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er, uint32_t& ev_out,
-                                          float4* sp, float* sv, const bool act, const int lane, const int N,
-                                          const int sbase, const int e, const int d, const float4 a,
+__device__ __forceinline__ void step_body(const int W, const Consts& c, const Dev& dv, Drone& s, EnvRegs& er,
+                                          uint32_t& ev_out, float4* sp, float* sv, const bool act, const int lane,
+                                          const int N, const int sbase, const int e, const int d, const float4 a,
                                           float* __restrict__ obs, float* __restrict__ rew, uint8_t* __restrict__ done,
-                                          const int observe_only, GoalCache& gc, const RowMap& rm, float* rows, const bool bulk) {
+                                          const int observe_only, GoalCache& gc, const RowMap& rm, float* rows,
+                                          const bool bulk) {
     const int nt = blockDim.x;
     const int K = c.K;
     const int keff = min(K, N - 1);
@@ -318,7 +321,8 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         fh[3] = command(c, a.w);
         const float u[4] = {sqrt_approx(fh[0]), sqrt_approx(fh[1]), sqrt_approx(fh[2]), sqrt_approx(fh[3])};
         const float zero3[3] = {0.f, 0.f, 0.f};
-        for (int sub = 0; sub < c.substeps; ++sub) ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, tick, d, sub, zero3);
+        for (int sub = 0; sub < c.substeps; ++sub)
+            ev |= substep<false, EXT == 2 ? 1 : 0>(s, er.p, c, u, tick, d, sub, zero3);
     }
 
     // ---- pair pass: collisions (S9, S10) and K nearest neighbours (S11)
@@ -337,8 +341,8 @@ __device__ __forceinline__ void step_body(const int W, const Consts& c, const De
         if (act && N > 1) {
             const bool coll = (c.flags & QS_F_COLLISIONS) && EXT != 2 && !observe_only;
             const bool flag_coll = (c.flags & QS_F_COLLISIONS) && !observe_only;
-            responded = pair_scan<(EXT > 0)>(c, s, er.p.thr, lane, N, sbase, sp, sv, nt, keff, coll, flag_coll, ev, nbrs, dvs,
-                                       dw && !observe_only, dw_az, dw_hit);
+            responded = pair_scan<(EXT > 0)>(c, s, er.p.thr, lane, N, sbase, sp, sv, nt, keff, coll, flag_coll, ev,
+                                             nbrs, dvs, dw && !observe_only, dw_az, dw_hit);
         }
         if (responded) apply_response(c, s, tick, d, dvs);
         if (dw && dw_hit && !observe_only) apply_downwash(c, s, tick, d, dw_az);
@@ -448,8 +452,9 @@ __device__ __forceinline__ SlotMap map_slot(const Dev& dv, const Tile& tile, con
 // wait costs more than the launch (1,048,576: 83.2 -> 87.9 us).
 constexpr int STEP_OVERLAP_WAVES = 2;
 template <int W, int EXT, bool OVERLAP = true, bool ROWS = (W == 1 && !EXT)>
-__global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
-                                                    const int* __restrict__ perm, const StepIO io, const int observe_only) {
+__global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168)
+    k_step(const Consts c, const Dev dv, const Tile* __restrict__ tiles, const int* __restrict__ perm, const StepIO io,
+           const int observe_only) {
     extern __shared__ float4 sm[];
     const SlotMap m = map_slot(dv, tile_at(dv, tiles, blockIdx.x, blockDim.x), perm, W);
     if (OVERLAP) await_previous();
@@ -469,8 +474,8 @@ __global__ void __maxnreg__(W == 1 ? 80 : W <= 32 && !EXT ? 96 : 168) k_step(con
     // counts: 1,048,576 81.0 and 80.5), or stored by the lanes (lane_rows)
     const RowMap rm = ROWS ? map_rows(m.act, m.d, 1, c.obs_dim) : RowMap();
     float* rows = reinterpret_cast<float*>(sm) + (threadIdx.x & ~31) * (c.obs_dim + ROW_PAD);
-    step_body<EXT, ROWS>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a, io.obs,
-              io.rew, io.done, observe_only, gc, rm, rows, io.bulk);
+    step_body<EXT, ROWS>(W, c, dv, s, er, ev, sm, reinterpret_cast<float*>(sm + blockDim.x), m.act, m.lane, m.N,
+                         m.sbase, m.e, m.d, a, io.obs, io.rew, io.done, observe_only, gc, rm, rows, io.bulk);
     if (m.act && !observe_only) {
         dv.ev[m.d] = ev;
         store_drone(s, dv.st, dv.D, m.d);
@@ -508,9 +513,10 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
         const float4 a = a_next;
         if (m.act && t + 1 < t0 + nsteps) a_next = *(act4 + (size_t)(t + 1) * D);
         float4* sp = sm + ((t - t0) & 1) * (SMEM_PLANES / 4) * blockDim.x;
-        step_body<EXT, !W1>(W, c, dv, s, er, ev, sp, reinterpret_cast<float*>(sp + blockDim.x), m.act, m.lane, m.N, m.sbase, m.e, m.d, a,
-                       io.obs ? io.obs + (size_t)t * D * c.obs_dim : nullptr, io.rew ? io.rew + (size_t)t * D : nullptr,
-                       io.done ? io.done + (size_t)t * E : nullptr, 0, gc, rm, rows, io.bulk);
+        step_body<EXT, !W1>(W, c, dv, s, er, ev, sp, reinterpret_cast<float*>(sp + blockDim.x), m.act, m.lane, m.N,
+                            m.sbase, m.e, m.d, a, io.obs ? io.obs + (size_t)t * D * c.obs_dim : nullptr,
+                            io.rew ? io.rew + (size_t)t * D : nullptr, io.done ? io.done + (size_t)t * E : nullptr, 0,
+                            gc, rm, rows, io.bulk);
     }
     if (!W1 && rm.lead) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
     if (m.act) {
@@ -536,10 +542,10 @@ __device__ __forceinline__ void rollout_tile(const Consts& c, const Dev& dv, con
 // 8% (34,000 drones, 32 steps: 102 us before the rows went that way, 111 after,
 // 96 in this instance, whose lanes store their own; 300,000 drones 579, 589, 532).
 template <int EXT, bool W1>
-__global__ void __maxnreg__(W1 && !EXT ? 104 : 128) k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
-                                                       const int n_tiles, const int* __restrict__ perm,
-                                                       int* __restrict__ counter, const RolloutIO io, const int t0,
-                                                       const int nsteps) {
+__global__ void __maxnreg__(W1 && !EXT ? 104 : 128)
+    k_rollout(const Consts c, const Dev dv, const Tile* __restrict__ tiles, const int n_tiles,
+              const int* __restrict__ perm, int* __restrict__ counter, const RolloutIO io, const int t0,
+              const int nsteps) {
     extern __shared__ float4 sm[];
     __shared__ int s_next;
     await_previous();
@@ -755,8 +761,8 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         if (act && N > 1) {
             const bool coll = (c.flags & QS_F_COLLISIONS) && EXT != 2;
             const bool flag_coll = (c.flags & QS_F_COLLISIONS) != 0;
-            responded = pair_scan<(EXT > 0)>(c, s, er.p.thr, lane, N, sbase, sh.sp, &sh.sv[0][0], 32 * P, keff, coll, flag_coll,
-                                       ev, nbrs, dvs, dw, dw_az, dw_hit);
+            responded = pair_scan<(EXT > 0)>(c, s, er.p.thr, lane, N, sbase, sh.sp, &sh.sv[0][0], 32 * P, keff, coll,
+                                             flag_coll, ev, nbrs, dvs, dw, dw_az, dw_hit);
         }
         if (responded) apply_response(c, s, er.tick, d, dvs);
         if (dw && dw_hit) apply_downwash(c, s, er.tick, d, dw_az);
@@ -895,8 +901,8 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
         __syncthreads();  // B2
         launch_next();
         if (io.obs)
-            ws_finish<1>(c, sh, m, map_rows(m.act, m.d, m.W, c.obs_dim), ws_rows(c, m.L), 0, io.obs, nullptr, false, ex, evv, ew,
-                         [](float*) {});
+            ws_finish<1>(c, sh, m, map_rows(m.act, m.d, m.W, c.obs_dim), ws_rows(c, m.L), 0, io.obs, nullptr, false,
+                         ex, evv, ew, [](float*) {});
         return;
     }
     // ---------------- dynamics warp
@@ -929,9 +935,9 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
 // 4864 / 2432 envs: +2% / +5% / +7%); swarm slots meet at B1 and B2 of every
 // step (without B1, 3.56e9 -> 3.50e9 quadrotor-steps/s for 2048 x 8).
 template <int EXT, int P>
-__global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1)) k_rollout_ws(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
-                                                       const int* __restrict__ perm, const RolloutIO io, const int t0,
-                                                       const int nsteps) {
+__global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : 1))
+    k_rollout_ws(const Consts c, const Dev dv, const Tile* __restrict__ tiles, const int* __restrict__ perm,
+                 const RolloutIO io, const int t0, const int nsteps) {
     __shared__ WsShared<P> sh;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, 32 * P);
     const WsMap m = ws_map<P>(dv, tile, perm);
@@ -1120,8 +1126,9 @@ __device__ __forceinline__ unsigned long long serve_wait(unsigned long long* go,
 // Left to itself the 64-lane common instance takes 193, two CTAs an SM; held to
 // three it fits in 144 without a spill (the general ones take 208 and 226).
 template <int EXT, int P>
-__global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : EXT == 0 ? 3 : 2)) k_serve(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
-                                                                  const int* __restrict__ perm, const ServeIO io, const int k0) {
+__global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : EXT == 0 ? 3 : 2))
+    k_serve(const Consts c, const Dev dv, const Tile* __restrict__ tiles, const int* __restrict__ perm, const ServeIO io,
+            const int k0) {
     __shared__ WsShared<P> sh;
     __shared__ unsigned long long s_go;
     const Tile tile = tile_at(dv, tiles, blockIdx.x, 32 * P);
@@ -1158,7 +1165,8 @@ __global__ void __launch_bounds__(64 * P, (P == 1 ? 6 : EXT == 0 ? 3 : 2)) k_ser
             float ex[3] = {0.f, 0.f, 0.f}, evv[3] = {0.f, 0.f, 0.f}, ew[3] = {0.f, 0.f, 0.f};
             if (m.act && io.obs && (c.flags & QS_F_OBS_NOISE)) obs_noise(c, tick, m.d, 0u, ex, evv, ew);
             __syncthreads();  // B2
-            if (io.obs) ws_finish<P>(c, sh, m, rm, ws_rows(c, m.L), b, io.obs, nullptr, false, ex, evv, ew, [](float*) {});
+            if (io.obs)
+                ws_finish<P>(c, sh, m, rm, ws_rows(c, m.L), b, io.obs, nullptr, false, ex, evv, ew, [](float*) {});
             ws_motor_normals<P>(c, sh, m, tick + 1, b ^ 1);
         } else {
             // the host's commands of this step: fetched again, never from a cached line
@@ -1237,7 +1245,8 @@ int rollout_ws_resident_ctas(const Consts& c, int P) {
 // CTAs with many neighbours) asks for the most any shape needs, so that no
 // handle's call lowers another's.
 cudaError_t allow_smem(const void* fn, size_t smem) {
-    return smem <= 48u << 10 ? cudaSuccess : cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM_MAX);
+    if (smem <= 48u << 10) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, STEP_SMEM_MAX);
 }
 
 // CTAs of `block` threads of the single-drone step (80 registers) in a wave.
@@ -1290,10 +1299,10 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
                         const StepIO& io, int observe_only, cudaStream_t st) {
     if (cp.n_tiles == 0) return cudaSuccess;
     const int ext = extended(c);
-    if (cp.ws && !observe_only)
-        return launch_overlapped(ext == 2 ? k_step_ws<2> : ext == 1 ? k_step_ws<1> : cp.W == 1 ? k_step_ws<0, true> : k_step_ws<0>, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv,
-                                 tiles + cp.tile_off,
-                                 perm, io);
+    if (cp.ws && !observe_only) {
+        const auto k = ext == 2 ? k_step_ws<2> : ext == 1 ? k_step_ws<1> : cp.W == 1 ? k_step_ws<0, true> : k_step_ws<0>;
+        return launch_overlapped(k, cp.n_tiles, 64, io.obs ? ws_smem(c, 1) : 0, st, c, dv, tiles + cp.tile_off, perm, io);
+    }
     const size_t smem = cp.W > 1 ? sizeof(float) * SMEM_PLANES * cp.block
                         : ext     ? 0
                                   : sizeof(float) * cp.block * (c.obs_dim + ROW_PAD);
