@@ -501,9 +501,9 @@ __global__ void __launch_bounds__(ADJ_BLOCK_MAX) k_diff_fwd(const Consts c, cons
 // next saved input instead of drawing it again.
 //
 // Bound by the chain of the reverse substeps with one warp of each group a
-// scheduler (1024 x 8 drones, 128 steps: forward 532 -> 382 us and reverse 646
-// -> 466 us with the near pairs and the room's faces tested ahead of their rare
-// branches and commands loaded a step ahead).
+// scheduler (1024 x 8 drones, 128 steps: forward 520 -> 362 us and reverse 667
+// -> 465 us with the near pairs tested ahead of their rare branch, forward the
+// room's faces too, and commands loaded a step ahead).
 // DENSE: 64-thread CTAs held to 168 registers (a few spills), six an SM
 // instead of four, for batches of several waves (dense_backward()).
 template <bool DENSE>

@@ -778,7 +778,7 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
         sh.rw[b][1][L] = make_float4(s.R[4], s.R[5], s.R[6], s.R[7]);
         sh.rw[b][2][L] = make_float4(s.R[8], s.w[0], s.w[1], s.w[2]);
         sh.gk[b][L] = make_float4(gl[0], gl[1], gl[2], __int_as_float(W > 1 ? keff : 0));
-        sh.nb[b][L] = nbrs + (NbrList)sbase * 0x0101010101010101ull;  // (fields past keff are not read)
+        if (!W1) sh.nb[b][L] = nbrs + (NbrList)sbase * 0x0101010101010101ull;  // (fields past keff are not read)
         if (DEFER) {  // the noise side computes the reward from these
             sh.fh[b][L] = make_float4(fh[0], fh[1], fh[2], fh[3]);
             sh.fp[b][L] = make_float4(s.fp[0], s.fp[1], s.fp[2], s.fp[3]);
@@ -805,10 +805,11 @@ __device__ __forceinline__ void ws_dynamics_step(const Consts& c, const Dev& dv,
 // Noise side: finishes the step published in buffer b. The observation rows
 // (with sensor noise ex, evv, ew) go to obs, and with rew the reward (the same
 // compute_reward as the dynamics side) of the lane's drone; goal(gl) replaces
-// the published single goal where scenarios are on. Every thread of the side
-// calls it. The rows took two thirds of the noise side's time, word by word:
+// the published single goal where scenarios are on; without BULK the rows are
+// always stored by the lanes, at once (one step: nothing to wait for). Every
+// thread of the side calls it. The rows took two thirds of the noise side's time, word by word:
 // 3,800 of 7,200 cycles a step for swarms of 8 at K = 6 (two CTAs an SM).
-template <int P, class Goal>
+template <int P, bool BULK = true, class Goal>
 __device__ __forceinline__ void ws_finish(const Consts& c, WsShared<P>& sh, const WsMap& m, const RowMap& rm, float* rows,
                                           int b, float* __restrict__ obs, float* __restrict__ rew, bool bulk,
                                           const float ex[3], const float evv[3], const float ew[3], const Goal& goal) {
@@ -831,7 +832,7 @@ __device__ __forceinline__ void ws_finish(const Consts& c, WsShared<P>& sh, cons
     }
     goal(gl);
     if (obs) {
-        rows_free(rm);
+        if (BULK) rows_free(rm);
         if (m.act) {
             float2* o2 = reinterpret_cast<float2*>(rows + rm.off + row_shift(rm, obs, od) + rm.rank * od);
             o2[0] = make_float2(s.x[0] - gl[0] + ex[0], s.x[1] - gl[1] + ex[1]);
@@ -861,7 +862,7 @@ __device__ __forceinline__ void ws_finish(const Consts& c, WsShared<P>& sh, cons
                 }
             }
         }
-        send_rows(rm, rows, obs, od, bulk);
+        send_rows(rm, rows, obs, od, BULK && bulk);
     }
     if (rew && m.act) {
         const float4 f = sh.fh[b][L], p = sh.fp[b][L];
@@ -882,8 +883,12 @@ __device__ __forceinline__ float* ws_rows(const Consts& c, int L) {
 }
 
 // W1: every slot of the launch holds one drone (no pair pass: a smaller kernel to
-// fetch when its instructions are cold; 8192 drones with L2 flushed before each
-// step 9.7 -> 9.1 us).
+// fetch when its instructions are cold). 8192 drones with L2 flushed before each
+// step, where the fetch counts (means of processes, each a mix of modes 0.3 - 1
+// us apart; sources that differ elsewhere in the library give 8.7 - 10.0 for the
+// same kernel): 9.75 us without W1, 9.05 - 9.25 with it, 8.7 - 9.2 with the rows
+// mapped ahead of B2 and no bulk-copy code in the step. Back to back in a stream
+// 4.0 -> 3.8 (4.4 before launches overlapped).
 template <int EXT, bool W1 = false>
 __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, const Tile* __restrict__ tiles,
                                                 const int* __restrict__ perm, const StepIO io) {
@@ -898,11 +903,11 @@ __global__ void __launch_bounds__(64) k_step_ws(const Consts c, const Dev dv, co
         __syncthreads();  // B1
         float ex[3] = {0.f, 0.f, 0.f}, evv[3] = {0.f, 0.f, 0.f}, ew[3] = {0.f, 0.f, 0.f};
         if (m.act && io.obs && (c.flags & QS_F_OBS_NOISE)) obs_noise(c, tick, m.d, 0u, ex, evv, ew);
+        const RowMap rm = map_rows(m.act, m.d, m.W, c.obs_dim);  // while the dynamics run
         __syncthreads();  // B2
         launch_next();
         if (io.obs)
-            ws_finish<1>(c, sh, m, map_rows(m.act, m.d, m.W, c.obs_dim), ws_rows(c, m.L), 0, io.obs, nullptr, false,
-                         ex, evv, ew, [](float*) {});
+            ws_finish<1, false>(c, sh, m, rm, ws_rows(c, m.L), 0, io.obs, nullptr, false, ex, evv, ew, [](float*) {});
         return;
     }
     // ---------------- dynamics warp
