@@ -335,7 +335,7 @@ qs_status upload_tiles(qs_env* h) {
     h->d_wtiles = h->d_tiles + n0 + n1 + n2;
     h->n_wtiles = (int)wtiles.size();
     h->single_drone = maxW == 1;
-    h->rollout_grid = rollout_grid(h->c, rblock, h->single_drone);
+    h->rollout_grid = rollout_grid(h->c, h->dv.D, rblock, h->single_drone);
     return QS_OK;
 }
 

@@ -186,8 +186,8 @@ int serve_resident_ctas(const Consts& c, int P);
 // resident at once.
 int rollout_ws_resident_ctas(const Consts& c, int P);
 // CTAs of `block` threads the device keeps resident at once for the k_rollout
-// instance launch_rollout picks (single: one drone per env).
-int rollout_grid(const Consts& c, int block, bool single);
+// instance launch_rollout picks (D drones; single: one drone per env).
+int rollout_grid(const Consts& c, int D, int block, bool single);
 
 // differentiable rollout (qs_adjoint.cu)
 size_t diff_workspace_bytes(int D, int T, int C, int substeps);

@@ -1318,17 +1318,27 @@ cudaError_t launch_step(const Consts& c, const Dev& dv, const ClassPlan& cp, con
 }
 
 // Whether a handle's rollout takes the single-drone form of its instance (the
-// common and the smooth one have it): every env holds one drone, and the row is
-// short, so that its lane had better store it than send it through shared memory.
-// Measured with one drone an env and K neighbour fields, us, stored by the lane
-// against sent: common 30,000 drones, 16 steps K = 1 47 and 54, K = 2 51 and 55,
-// K = 6 81 and 58; 100,000, 12 steps K = 2 115 and 92, K = 6 270 and 96; smooth
-// 30,000 K = 2 54 and 61, 100,000 K = 1 91 and 106, K = 6 245 and 112.
-bool single_form(const Consts& c, bool single) { return single && extended(c) != 1 && c.K <= 2; }
+// common and the smooth one have it): every env holds one drone, and the rows'
+// neighbour fields are few enough that a lane had better store its own row than
+// send it through shared memory, whose addressing costs a step more but whose
+// stores do not scatter. Measured with one drone an env, us for 12 steps, stored
+// by the lane against sent: K = 3 24,000 drones 40 and 43, 32,000 48 and 43; K = 6
+// 12,000 35 and 39, 16,384 39 and 39, 20,000 49 and 43, 100,000 270 and 96; K = 8
+// 12,000 37 and 39, 16,384 45 and 40; smooth K = 6 16,384 38 and 43, 20,000 51 and
+// 48. With K = 1 the lane's stores win at every size (1,048,576 drones, 4 steps 218
+// and 226).
+bool single_form(const Consts& c, int D, bool single) {
+    if (!single || extended(c) == 1) return false;
+    if (c.K < 2) return true;
+    int dev = 0, n_sm = 152;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    return (long)D * c.K <= 640L * n_sm;
+}
 
-// The k_rollout instance for a handle.
-auto rollout_kernel(const Consts& c, bool single) {
-    const bool form = single_form(c, single);
+// The k_rollout instance for a handle of D drones.
+auto rollout_kernel(const Consts& c, int D, bool single) {
+    const bool form = single_form(c, D, single);
     switch (extended(c)) {
         case 2: return form ? k_rollout<2, true> : k_rollout<2, false>;
         case 1: return k_rollout<1, false>;
@@ -1338,17 +1348,17 @@ auto rollout_kernel(const Consts& c, bool single) {
 
 // Its dynamic shared memory: goal values (general instances) and, but for the
 // single-drone forms, two sets of staging planes and the CTA's observation rows.
-size_t rollout_smem(const Consts& c, int block, bool single) {
+size_t rollout_smem(const Consts& c, int D, int block, bool single) {
     const int goal = extended(c) ? GOAL_STRIDE : 0;
-    return sizeof(float) * block * (single_form(c, single) ? goal : 2 * SMEM_PLANES + goal + c.obs_dim + ROW_PAD);
+    return sizeof(float) * block * (single_form(c, D, single) ? goal : 2 * SMEM_PLANES + goal + c.obs_dim + ROW_PAD);
 }
 
-int rollout_grid(const Consts& c, int block, bool single) {
+int rollout_grid(const Consts& c, int D, int block, bool single) {
     int dev = 0, n_sm = 0, occ = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    const void* fn = (const void*)rollout_kernel(c, single);
-    const size_t smem = rollout_smem(c, block, single);
+    const void* fn = (const void*)rollout_kernel(c, D, single);
+    const size_t smem = rollout_smem(c, D, block, single);
     allow_smem(fn, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, block, smem);
     return (occ > 0 ? occ : 1) * n_sm;
@@ -1368,8 +1378,8 @@ cudaError_t launch_rollout_ws(const Consts& c, const Dev& dv, const Tile* tiles,
 cudaError_t launch_rollout(const Consts& c, const Dev& dv, const Tile* tiles, int n_tiles, int block, const int* perm,
                            int* counter, const RolloutIO& io, int t0, int nsteps, int grid, bool single,
                            cudaStream_t st) {
-    const size_t smem = rollout_smem(c, block, single);
-    const auto k = rollout_kernel(c, single);
+    const size_t smem = rollout_smem(c, dv.D, block, single);
+    const auto k = rollout_kernel(c, dv.D, single);
     const cudaError_t e = allow_smem((const void*)k, smem);
     if (e != cudaSuccess) return e;
     const int g = grid > 0 ? grid : n_tiles;

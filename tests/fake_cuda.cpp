@@ -108,6 +108,6 @@ cudaError_t launch_goals(const Consts&, const Dev&, float*, cudaStream_t) { retu
 cudaError_t launch_check_selftest(const Dev&, int, cudaStream_t) { return launch(); }
 int serve_resident_ctas(const Consts&, int P) { return 152 * 6 / P; }
 int rollout_ws_resident_ctas(const Consts&, int P) { return 152 * 6 / P; }
-int rollout_grid(const Consts&, int, bool) { return 152; }
+int rollout_grid(const Consts&, int, int, bool) { return 152; }
 size_t diff_workspace_bytes(int, int, int, int) { return 256; }
 }  // namespace qsk

@@ -1,6 +1,7 @@
 """Rows of single-drone handles in the persistent rollout: stored by their lanes
-while short (K <= 2), sent through shared memory beyond, both equal to per-call
-steps wherever the buffer starts, with nothing written around them."""
+while their neighbour fields are few (up to 640 an SM in all), sent through shared
+memory beyond, both equal to per-call steps wherever the buffer starts, with
+nothing written around them."""
 import pytest
 import torch
 
@@ -18,6 +19,18 @@ FEATS = {"common": ("floor", "walls", "motor_noise", "obs_noise", "dr"), "smooth
 @pytest.mark.parametrize("E,block,where", [(1, 32, "aligned"), (31, 32, "offset"), (33, 64, "pinned"), (1537, 32, "pinned"),
                                            (1537, 128, "offset"), (700, 256, "aligned")])
 def test_rows_equal_steps(feats, K, E, block, where):
+    check(feats, K, E, block, where)
+
+
+@pytest.mark.parametrize("feats", ["common", "smooth"])
+@pytest.mark.parametrize("K,block,where", [(1, 32, "offset"), (2, 32, "aligned"), (3, 64, "offset"), (8, 32, "pinned"),
+                                           (8, 128, "offset"), (6, 256, "aligned")])
+@pytest.mark.parametrize("past", [0, 1])
+def test_both_sides_of_the_line(feats, K, block, where, past):
+    check(feats, K, 640 * torch.cuda.get_device_properties(DEV).multi_processor_count // K + past, block, where)
+
+
+def check(feats, K, E, block, where):
     T = 3
     a, b = (QuadSwarmEnv(E, 1, K, FEATS[feats], seed=4, device=DEV) for _ in range(2))
     qs.qs_set_rollout_shape(a.h, block, 0, False)
