@@ -58,7 +58,10 @@ cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { return cudaMalloc(p, n
 cudaError_t cudaFreeHost(void* p) { return cudaFree(p); }
 cudaError_t cudaHostGetDevicePointer(void** d, void* p, unsigned) { *d = p; return cudaSuccess; }
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) { memcpy(d, s, n); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+    memcpy(d, s, n);
+    return cudaSuccess;
+}
 cudaError_t cudaMemset(void* p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void* p, int v, size_t n, cudaStream_t) { memset(p, v, n); return cudaSuccess; }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
@@ -86,26 +89,44 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
     *g = g_invalid ? nullptr : (cudaGraph_t)(size_t)g_captures;
     return g_invalid ? ret(cudaErrorStreamCaptureInvalidated) : cudaSuccess;
 }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long) { *e = (cudaGraphExec_t)g; return cudaSuccess; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long) {
+    *e = (cudaGraphExec_t)g;
+    return cudaSuccess;
+}
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { ++g_replays; return cudaSuccess; }
 }
 
 namespace qsk {
-cudaError_t launch_step(const Consts&, const Dev&, const ClassPlan&, const Tile*, const int*, const StepIO&, int, cudaStream_t) { return launch(); }
-cudaError_t launch_rollout(const Consts&, const Dev&, const Tile*, int, int, const int*, int*, const RolloutIO& io, int, int, int, bool, cudaStream_t) { return rollout(io); }
-cudaError_t launch_rollout_ws(const Consts&, const Dev&, const Tile*, int, int, const int*, const RolloutIO& io, int, int, cudaStream_t) { return rollout(io); }
-cudaError_t launch_serve(const Consts&, const Dev&, const Tile*, int, int, const int*, const ServeIO&, int, cudaStream_t) { return launch(); }
-cudaError_t launch_diff(int, const Consts&, const Dev&, const Tile*, int, int, const int*, const float*, const float*, float*, const float*, float*, float*, void*, int, int, cudaStream_t) { return launch(); }
-cudaError_t launch_philox(const uint32_t*, uint32_t, uint32_t, int, uint32_t*, long long, cudaStream_t) { return launch(); }
-cudaError_t launch_reset(const Consts&, const Dev&, uint32_t, uint32_t, const uint8_t*, cudaStream_t) { return launch(); }
-cudaError_t launch_get_state(const Dev&, float*, float*, float*, int32_t*, uint32_t*, cudaStream_t) { return launch(); }
-cudaError_t launch_set_state(const Consts&, const Dev&, const float*, const float*, const float*, const int32_t*, const uint32_t*, cudaStream_t) { return launch(); }
-cudaError_t launch_get_events(const Dev&, int, uint32_t*, int16_t*, cudaStream_t) { return launch(); }
-cudaError_t launch_scenario_io(const Dev&, float*, const float*, cudaStream_t) { return launch(); }
-cudaError_t launch_goals(const Consts&, const Dev&, float*, cudaStream_t) { return launch(); }
-cudaError_t launch_check_selftest(const Dev&, int, cudaStream_t) { return launch(); }
+typedef cudaError_t E;
+typedef cudaStream_t S;
+E launch_step(const Consts&, const Dev&, const ClassPlan&, const Tile*, const int*, const StepIO&, int, S) {
+    return launch();
+}
+E launch_rollout(const Consts&, const Dev&, const Tile*, int, int, const int*, int*, const RolloutIO& io, int, int, int,
+                 bool, S) {
+    return rollout(io);
+}
+E launch_rollout_ws(const Consts&, const Dev&, const Tile*, int, int, const int*, const RolloutIO& io, int, int, S) {
+    return rollout(io);
+}
+E launch_serve(const Consts&, const Dev&, const Tile*, int, int, const int*, const ServeIO&, int, S) { return launch(); }
+E launch_diff(int, const Consts&, const Dev&, const Tile*, int, int, const int*, const float*, const float*, float*,
+              const float*, float*, float*, void*, int, int, S) {
+    return launch();
+}
+E launch_philox(const uint32_t*, uint32_t, uint32_t, int, uint32_t*, long long, S) { return launch(); }
+E launch_reset(const Consts&, const Dev&, uint32_t, uint32_t, const uint8_t*, S) { return launch(); }
+E launch_get_state(const Dev&, float*, float*, float*, int32_t*, uint32_t*, S) { return launch(); }
+E launch_set_state(const Consts&, const Dev&, const float*, const float*, const float*, const int32_t*,
+                   const uint32_t*, S) {
+    return launch();
+}
+E launch_get_events(const Dev&, int, uint32_t*, int16_t*, S) { return launch(); }
+E launch_scenario_io(const Dev&, float*, const float*, S) { return launch(); }
+E launch_goals(const Consts&, const Dev&, float*, S) { return launch(); }
+E launch_check_selftest(const Dev&, int, S) { return launch(); }
 int serve_resident_ctas(const Consts&, int P) { return 152 * 6 / P; }
 int rollout_ws_resident_ctas(const Consts&, int P) { return 152 * 6 / P; }
 int rollout_grid(const Consts&, int, int, bool) { return 152; }
